@@ -17,8 +17,8 @@
 // cells included; here a ring cell's slots may already hold its owner's
 // post-collision values).  The step stages phi of three planes (tile and
 // ring) from that array and the tile's own g one plane ahead; the per-cell
-// arithmetic is that of the two-set kernels (phase-field outputs first, the
-// moment differences parked in the consumed g column), so the results equal
+// arithmetic is that of the two-set kernels (here the phase-field outputs first,
+// then the relaxation and the flow), so the results equal
 // them to within the rounding of separately compiled units.
 #define LBMP_TILE_NS tile_aa
 #define LBMP_FUSED_MINB 3
@@ -143,16 +143,14 @@ __device__ __forceinline__ void collide_cell(const DevParams& p, const AAPtrs& D
             const int cz = Lat<3>::cz(a);
             return (cz < 0 ? pm : (cz == 0 ? pc : pn))[Lat<3>::cy(a) * RX + Lat<3>::cx(a)];
         },
-        centre, grad, lap);
+        grad, lap);
     CellState s;
     float inv_rho, nu;
     flow_closure<3>(p, centre.x, grad, lap, m, s, inv_rho, nu);
     phase_outputs<3>(p, s, GFromStrided{gcol, NT}, centre.x, centre.y, AAOut<Odd, Walls>{D.g, own, P});
-    float dh[27];
-    flow_relax<3>(m, s, inv_rho, nu, dh);
-#pragma unroll
-    for (int a = 0; a < Q3; ++a) gcol[a * NT] = dh[a];
-    flow_outputs<3>(s, DhStrided{gcol, NT}, m, AAOut<Odd, Walls>{D.f, own, P});
+    Residual R;
+    flow_relax<3>(m, s, inv_rho, nu, R);
+    flow_outputs<3>(p, s, R, m, AAOut<Odd, Walls>{D.f, own, P});
 }
 
 // planes [z0, z1) of the tile at (x0, y0); ends with a barrier

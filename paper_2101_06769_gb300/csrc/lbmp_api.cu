@@ -105,6 +105,7 @@ void fill_devparams(lbmp_handle* h)
     q.rho_l = (float)d.rho_l;
     q.drho = (float)(d.rho_h - d.rho_l);
     q.rho_bar = (float)(0.5 * (d.rho_h + d.rho_l));
+    q.drho6 = (float)((d.rho_h - d.rho_l) / 6.0);
     q.nu_h = (float)d.nu_h;
     q.nu_l = (float)d.nu_l;
     q.eta_h = (float)(d.rho_h * d.nu_h);
@@ -112,10 +113,15 @@ void fill_devparams(lbmp_handle* h)
     q.beta2 = (float)(2.0 * d.beta);
     q.kappa = (float)d.kappa;
     q.inv_tau_phi = (float)(1.0 / d.tau_phi);
+    q.neg_inv_tau = -q.inv_tau_phi;
     q.lam_sharp = (float)(d.lambda_phi * 4.0 / d.W);
-    q.lam_corr = (float)(d.lambda_phi * ((h->reduced && h->D == 3) ? 4.0 : 3.0));
+    q.lam_n = (float)(d.tau_phi * d.lambda_phi * 4.0 / d.W);
+    q.lam_corr = (float)(d.tau_phi * d.lambda_phi * ((h->reduced && h->D == 3) ? 4.0 : 3.0));
     q.g_accel = (float)d.g_accel;
     q.force_x = (float)d.force_x;
+    const bool uniform = (h->params.flags & LBMP_FLAG_UNIFORM_FORCE) != 0;
+    q.grav_h = uniform ? 0.f : (float)(0.5 * d.g_accel);
+    q.force_xh = uniform ? (float)(0.5 * d.force_x) : 0.f;
     q.flags = h->params.flags;
     q.wait_ns = 2000000000ull;  // 2 s
     q.test_extra_tx = 0;

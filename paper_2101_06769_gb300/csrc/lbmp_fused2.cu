@@ -245,15 +245,17 @@ __device__ __forceinline__ void fused2_segment(const DevParams& p, const DirPtrs
             float grad[3], lap;
             stencil_from_nb<2>(nh, nl, grad, lap);
             CellState s;
-            float dh[27];
-            flow_collide<2>(p, nh[4], grad, lap, m, s, dh);
+            float inv_rho, nu;
+            flow_closure<2>(p, nh[4], grad, lap, m, s, inv_rho, nu);
+            Residual Rs;
+            flow_relax<2>(m, s, inv_rho, nu, Rs);
             const off2 self = R.ys[1] + own.xs[1];
             if constexpr (PR)
-                collide_outputs<2, true>(p, s, DhArray{dh}, m, GFromStrided{gS + cur * QG * TX2 + tid, TX2}, nh[4],
+                collide_outputs<2, true>(p, s, Rs, m, GFromStrided{gS + cur * QG * TX2 + tid, TX2}, nh[4],
                                          nl[4], Out2{D.fout, self}, Out2{D.gout, self},
                                          PhiUStaged<2>{p, phiu, elem2(self), uS + cur * 2 * TX2 + tid, TX2});
             else
-                collide_outputs<2>(p, s, DhArray{dh}, m, GFromStrided{gS + cur * Q2 * TX2 + tid, TX2}, nh[4], nl[4],
+                collide_outputs<2>(p, s, Rs, m, GFromStrided{gS + cur * Q2 * TX2 + tid, TX2}, nh[4], nl[4],
                                    Out2{D.fout, self}, Out2{D.gout, self});
         }
     }

@@ -80,19 +80,6 @@ struct StageCopy {
 
 
 template <bool Walls>
-struct FCopy {
-    const DirPtrs& D;
-    const Column& C;
-    const Plane& P;
-    float* fbuf;
-    template <int a>
-    __device__ __forceinline__ void step() const
-    {
-        cp_async4(fbuf + a * NT, pulled<Walls, a>(D.fin, C, P));
-    }
-};
-
-template <bool Walls>
 struct RingCopy {
     const DirPtrs& D;
     const Column& C;
@@ -148,8 +135,8 @@ __device__ __forceinline__ void stage_issue(const DevParams& p, const DirPtrs& D
     }
     cp_async_commit();
     if constexpr (kRingReg) {
-        // the phi plane slot is free: the barrier ending the previous plane
-        // separates this write from the last stencil reads of its old plane
+        // the phi plane slot is free: it was last read before the previous
+        // plane's barrier
         if (tid < NRING) {
             if (P.lo || P.hi)
                 ring_phi_direct<true>(D, ring, P, phi_plane + rslot);
@@ -174,106 +161,73 @@ __device__ __forceinline__ void stage_finish(int tid, int oslot, int rslot, cons
 }
 
 // One segment of work: planes [z0, z1) of the tile at (x0, y0) of the domain
-// described by (p, Dp).  smem holds the g staging buffers, the ring buffer and
-// the three phi planes.  Ends with a barrier, so the caller may reuse shared
-// memory afterwards.
+// described by (p, Dp).  smem holds the g staging buffers, the ring buffer
+// and two phi planes.  One barrier per plane: every shared value but phi is
+// written and read by the same thread, and the phi of plane z+1 goes to the
+// slot that was last read before the previous plane's barrier.  Ends with a
+// barrier, so the caller may reuse shared memory afterwards.
 __device__ __forceinline__ void fused_segment(const DevParams& p, const DirPtrs& Dp, const ThreadGeo& T, float* smem,
                                               int x0, int y0, int z0, int z1, float* __restrict__ phiu)
 {
     float* gS = smem;                                    // [2][QG][NT]
     float* rS = smem + 2 * QG * NT;                      // [QG][NRING] ring cells' g of the plane being staged
-    float2* phiS = (float2*)(rS + (kRingReg ? 0 : QG * NRING));  // (hi, lo) [3][RY][RX]
-    float* fS = (float*)(phiS + 3 * PLANE);              // [27][NT] f' of the plane (LBMP_FUSED_FSMEM)
-    float* dS = fS + LBMP_FUSED_FSMEM * Q3 * NT;         // [27][NT] dh (kDhSmem)
-    float* uS = dS + (kDhSmem ? Q3 * NT : 0);            // [2][3][NT] previous phi u (reduced phase lattice)
+    float2* phiS = (float2*)(rS + (kRingReg ? 0 : QG * NRING));  // (hi, lo) [2][RY][RX]
+    float* uS = (float*)(phiS + 2 * PLANE);              // [2][3][NT] previous phi u (reduced phase lattice)
     const int tid = T.tid, oslot = T.oslot, rslot = T.rslot;
     Column own, ring;
     set_column(own, p, pmod(x0 + T.tx, p.nx), pmod(y0 + T.ty, p.ny));
     set_column(ring, p, pmod(x0 + T.lx, p.nx), pmod(y0 + T.ly, p.ny));
     const bool valid = (x0 + T.tx < p.nx) && (y0 + T.ty < p.ny);
-    int sP = 0, sC = 1, sN = 2;
-    stage_issue(p, Dp, own, ring, tid, rslot, z0 - 1, gS + QG * NT, rS, phiu, uS + 3 * NT, phiS + sP * PLANE);
-    stage_finish(tid, oslot, rslot, gS + QG * NT, rS, phiS + sP * PLANE);
-    stage_issue(p, Dp, own, ring, tid, rslot, z0, gS, rS, phiu, uS, phiS + sC * PLANE);
-    stage_finish(tid, oslot, rslot, gS, rS, phiS + sC * PLANE);
+    const auto layer = [&](int slot, LayerSums& L) {
+        const float2* c = phiS + slot * PLANE + oslot;
+        layer_sums<3>([&](int dx, int dy) { return c[dy * RX + dx]; }, L);
+    };
+    stage_issue(p, Dp, own, ring, tid, rslot, z0 - 1, gS + QG * NT, rS, phiu, uS + 3 * NT, phiS);
+    stage_finish(tid, oslot, rslot, gS + QG * NT, rS, phiS);
+    stage_issue(p, Dp, own, ring, tid, rslot, z0, gS, rS, phiu, uS, phiS + PLANE);
+    stage_finish(tid, oslot, rslot, gS, rS, phiS + PLANE);
+    LayerSums below, here;
+    __syncthreads();
+    layer(0, below);
+    layer(1, here);
+    __syncthreads();
     for (int z = z0; z < z1; ++z) {
         const int cur = (z - z0) & 1;
         // g(z+1) and the ring copies in flight while f'(z) is loaded
         stage_issue(p, Dp, own, ring, tid, rslot, z + 1, gS + (cur ^ 1) * QG * NT, rS, phiu, uS + (cur ^ 1) * 3 * NT,
-                    phiS + sN * PLANE);
+                    phiS + cur * PLANE);
         Plane P;
         set_plane(P, p, z);
         FlowMoments m;
-#if LBMP_FUSED_FSMEM
-        if (P.lo || P.hi)
-            Unroll<Q3>::run(FCopy<true>{Dp, own, P, fS + tid});
-        else
-            Unroll<Q3>::run(FCopy<false>{Dp, own, P, fS + tid});
-        cp_async_commit();
-        stage_finish(tid, oslot, rslot, gS + (cur ^ 1) * QG * NT, rS, phiS + sN * PLANE);
         {
             float fr[Q3];
-#pragma unroll
-            for (int a = 0; a < Q3; ++a) fr[a] = fS[a * NT + tid];
+            if (P.lo || P.hi)
+                Unroll<Q3>::run(PullLoad<true>{Dp.fin, own, P, fr});
+            else
+                Unroll<Q3>::run(PullLoad<false>{Dp.fin, own, P, fr});
+            stage_finish(tid, oslot, rslot, gS + (cur ^ 1) * QG * NT, rS, phiS + cur * PLANE);
             flow_moments<3>(m, fr);
         }
-#else
-        float fr[Q3];
-        if (P.lo || P.hi)
-            Unroll<Q3>::run(PullLoad<true>{Dp.fin, own, P, fr});
-        else
-            Unroll<Q3>::run(PullLoad<false>{Dp.fin, own, P, fr});
-        stage_finish(tid, oslot, rslot, gS + (cur ^ 1) * QG * NT, rS, phiS + sN * PLANE);
-        flow_moments<3>(m, fr);
-#endif
         __syncthreads();
+        LayerSums above;
+        layer(cur, above);
         if (valid) {
-            const float2* pm = phiS + sP * PLANE + oslot;
-            const float2* pc = phiS + sC * PLANE + oslot;
-            const float2* pn = phiS + sN * PLANE + oslot;
-            const float2 centre = pc[0];
             float grad[3], lap;
-            stencil_from<3>(
-                [&](int a) {
-                    const int cz = Lat<3>::cz(a);
-                    return (cz < 0 ? pm : (cz == 0 ? pc : pn))[Lat<3>::cy(a) * RX + Lat<3>::cx(a)];
-                },
-                centre, grad, lap);
+            stencil_from_layers<3>(below, here, above, grad, lap);
             CellState s;
+            float inv_rho, nu;
+            Residual R;
+            flow_closure<3>(p, here.c.x, grad, lap, m, s, inv_rho, nu);
             const cell_off self = P.zs[1] + own.ys[1] + own.xs[1];
-            float* gcol = gS + cur * QG * NT + tid;  // this cell's staged pre-collision g
-            if constexpr (kSplit) {
-                // g first; its staged column then holds the moment differences
-                float inv_rho, nu;
-                flow_closure<3>(p, centre.x, grad, lap, m, s, inv_rho, nu);
-                phase_outputs<3>(p, s, GFromStrided{gcol, NT}, centre.x, centre.y, CellOut{Dp.gout, self});
-                float dh[27];
-                flow_relax<3>(m, s, inv_rho, nu, dh);
-#pragma unroll
-                for (int a = 0; a < Q3; ++a) gcol[a * NT] = dh[a];
-                flow_outputs<3>(s, DhStrided{gcol, NT}, m, CellOut{Dp.fout, self});
-            } else {
-                float dh[27];
-                flow_collide<3>(p, centre.x, grad, lap, m, s, dh);
-                if constexpr (kDhSmem) {
-#pragma unroll
-                    for (int a = 0; a < Q3; ++a) dS[a * NT + tid] = dh[a];
-                    collide_outputs<3, PR>(p, s, DhStrided{dS + tid, NT}, m, GFromStrided{gcol, NT}, centre.x,
-                                           centre.y, CellOut{Dp.fout, self}, CellOut{Dp.gout, self},
-                                           PhiUStaged<3>{p, phiu, elem_index(self), uS + cur * 3 * NT + tid, NT});
-                } else {
-                    collide_outputs<3, PR>(p, s, DhArray{dh}, m, GFromStrided{gcol, NT}, centre.x, centre.y,
-                                           CellOut{Dp.fout, self}, CellOut{Dp.gout, self},
-                                           PhiUStaged<3>{p, phiu, elem_index(self), uS + cur * 3 * NT + tid, NT});
-                }
-            }
+            const GFromStrided gin{gS + cur * QG * NT + tid, NT};  // this cell's staged pre-collision g
+            flow_relax<3>(m, s, inv_rho, nu, R);
+            collide_outputs<3, PR>(p, s, R, m, gin, here.c.x, here.c.y, CellOut{Dp.fout, self}, CellOut{Dp.gout, self},
+                                   PhiUStaged<3>{p, phiu, elem_index(self), uS + cur * 3 * NT + tid, NT});
         }
-        __syncthreads();
-        const int t = sP;
-        sP = sC;
-        sC = sN;
-        sN = t;
+        below = here;
+        here = above;
     }
+    __syncthreads();
 }
 
 __global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_fused3_kernel(DevParams p, FusedArgs A, DirPtrs Dp)

@@ -181,7 +181,6 @@ __device__ __forceinline__ bool bulk_segment(const DevParams& p, const DirPtrs& 
 {
     float* gW = smem;                               // [2][WIN] staged windows
     float2* phiS = (float2*)(gW + 2 * WIN);         // (hi, lo) [3][RY][RX]
-    float* dS = (float*)(phiS + 3 * PLANE);         // [27][NT] dh (LBMP_FUSED_DHSMEM)
     const int tid = T.tid;
     Column own;
     set_column(own, p, pmod(x0 + T.tx, p.nx), pmod(y0 + T.ty, p.ny));
@@ -224,24 +223,19 @@ __device__ __forceinline__ bool bulk_segment(const DevParams& p, const DirPtrs& 
                     const int cz = Lat<3>::cz(a);
                     return (cz < 0 ? pm : (cz == 0 ? pc : pn))[Lat<3>::cy(a) * RX + Lat<3>::cx(a)];
                 },
-                centre, grad, lap);
+                grad, lap);
             CellState s;
-            float dh[27];
-            flow_collide<3>(p, centre.x, grad, lap, m, s, dh);
+            float inv_rho, nu;
+            flow_closure<3>(p, centre.x, grad, lap, m, s, inv_rho, nu);
+            Residual R;
+            flow_relax<3>(m, s, inv_rho, nu, R);
             const int self = P.zs[1] + own.ys[1] + own.xs[1];
             const float* wc = gW + cur * WIN;
-#if LBMP_FUSED_DHSMEM
-#pragma unroll
-            for (int a = 0; a < Q3; ++a) dS[a * NT + tid] = dh[a];
-            const DhStrided dsrc{dS + tid, NT};
-#else
-            const DhArray dsrc{dh};
-#endif
             if (P.lo || P.hi)
-                collide_outputs<3>(p, s, dsrc, m, GFromWin<true>{wc, T.ty + 1, T.tx + 4, P.lo, P.hi}, centre.x,
+                collide_outputs<3>(p, s, R, m, GFromWin<true>{wc, T.ty + 1, T.tx + 4, P.lo, P.hi}, centre.x,
                                    centre.y, PtrOut{Dp.fout, self}, PtrOut{Dp.gout, self});
             else
-                collide_outputs<3>(p, s, dsrc, m, GFromWin<false>{wc, T.ty + 1, T.tx + 4, false, false}, centre.x,
+                collide_outputs<3>(p, s, R, m, GFromWin<false>{wc, T.ty + 1, T.tx + 4, false, false}, centre.x,
                                    centre.y, PtrOut{Dp.fout, self}, PtrOut{Dp.gout, self});
         }
         __syncthreads();
@@ -292,7 +286,7 @@ bool bulk_supported(const lbmp_handle* h)
 
 cudaError_t launch_step_fused_bulk(lbmp_handle* h)
 {
-    const size_t smem = sizeof(float) * (2 * WIN + LBMP_FUSED_DHSMEM * Q3 * NT) + sizeof(float2) * 3 * PLANE;
+    const size_t smem = sizeof(float) * 2 * WIN + sizeof(float2) * 3 * PLANE;
     if (g_bulk.device != h->device) {
         cudaError_t e =
             cudaFuncSetAttribute(step_fused3b_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

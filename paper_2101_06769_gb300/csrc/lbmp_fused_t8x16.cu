@@ -1,15 +1,15 @@
 // lbmp_fused_t8x16.cu -- the fused D3Q27 FP32 step and its batch form at a
 // 8 x 16 tile (a launch shape of the autotuners; kernel source
 // lbmp_fused3_body.cuh).
-// Four CTAs (16 warps) per SM at 128 registers: the phase-field outputs
-// first, the moment differences parked in the consumed g column, ring phi
-// from register loads, pair loops kept in order (measured on the
-// 128x128x512 RT workload: 0.852 ms per step against 0.894 ms for three
-// CTAs per SM with a separate moment-difference array); column and plane
-// offsets in bytes (0.827 against 0.860 ms with element indices)
+// Four CTAs (16 warps) per SM at 128 registers, ring phi from register loads,
+// column and plane offsets in bytes.  On the 128x128x512 RT workload a step
+// takes 0.738 ms (0.820 ms with the earlier arithmetic, which issued 2334
+// instructions per cell, and two barriers per plane).  It no longer follows the
+// instruction count: 3 or 5 CTAs per SM take 0.747 / 0.745 ms, element indices
+// 0.732, a ring staged by cp.async 0.748, a 32 x 8 tile 0.778, and the same
+// access pattern without arithmetic 0.706 ms.
 #define LBMP_FUSED_MINB 4
 #define LBMP_FUSED_BYTEOFF 4
-#define LBMP_FUSED_SPLIT 1
 #define LBMP_FUSED_RINGREG 1
 #define LBMP_OUT_ORDERED 1
 #define LBMP_FUSED_TX 8

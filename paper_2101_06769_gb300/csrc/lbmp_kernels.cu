@@ -7,6 +7,7 @@
 // opposite population of the cell itself (Sec. 3.2 boundary treatment).
 #include <math.h>
 
+#include "lbmp_coded.cuh"
 #include "lbmp_internal.h"
 
 namespace lbmp {
@@ -104,28 +105,9 @@ __global__ void __launch_bounds__(128) step_simple_kernel(DevParams p, Pop<D, St
         nh[a] = phi[j];
         nl[a] = phi[p.N + j];
     }
-    float grad[3], lap;
-    stencil_from_nb<D>(nh, nl, grad, lap);
     float fr[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) fr[a] = pulled_value<D, St>(p, fin, a, x, y, z, i);
-    FlowMoments m;
-    flow_moments<D>(m, fr);
-    CellState s;
-    float dh[27];
-    if constexpr (!PR && !St::shifted) {
-        if (p.flags & kFlagDivU) {  // the w cs2 rho div(u) term of Xi (Sec. 2.3)
-            flow_collide<D, true>(p, nh[Q / 2], grad, lap, m, s, dh, div_stored<D>(p, us_in, x, y, z));
-            for (int k = 0; k < D; ++k) us_out[k * p.N + i] = s.u[k];
-            float gd[Q];
-#pragma unroll
-            for (int a = 0; a < Q; ++a) gd[a] = pulled_value<D, St>(p, gin, a, x, y, z, i);
-            collide_outputs<D, false, true>(p, s, DhArray{dh}, m, GFromArray{gd}, nh[Q / 2], nl[Q / 2],
-                                            SoAOut{fout.base + i, p.N}, SoAOut{gout.base + i, p.N});
-            return;
-        }
-    }
-    flow_collide<D>(p, nh[Q / 2], grad, lap, m, s, dh);
     constexpr int QG = PhaseLat<D, PR>::Q;
     float gr[QG];
 #pragma unroll
@@ -134,20 +116,45 @@ __global__ void __launch_bounds__(128) step_simple_kernel(DevParams p, Pop<D, St
         const long long c = pull_src_g<D, PR>(p, r, x, y, z, i, slot);
         gr[r] = gin.load(slot, c);
     }
-    if constexpr (PR) {
-        collide_outputs<D, true>(p, s, DhArray{dh}, m, GFromArray{gr}, nh[Q / 2], nl[Q / 2], SoAOut{fout.base + i, p.N},
-                                 SoAOut{gout.base + i, p.N}, PhiUStep<D>{p, phiu, i});
-    } else if constexpr (St::shifted) {
+    const float ph = nh[Q / 2], pl = nl[Q / 2];
+    float grad[3], lap, inv_rho, nu;
+    if constexpr (St::shifted) {
+        coded::stencil_from_nb<D>(nh, nl, grad, lap);
+        coded::FlowMoments m;
+        coded::flow_moments<D>(m, fr);
+        coded::CellState s;
+        float dh[27];
+        coded::flow_closure<D>(p, ph, grad, lap, m, s, inv_rho, nu);
+        coded::flow_relax<D>(m, s, inv_rho, nu, dh);
         float off_f, off_g;
-        rest_offsets<D, St>(p, s, dh, GFromArray{gr}, off_f, off_g);
-        collide_outputs<D>(p, s, DhArray{dh}, m, GFromArray{gr}, nh[Q / 2], nl[Q / 2],
-                           EncSoA<D, St>{fout.base + i, (unsigned short*)(fout.base + p.N) + i, p.N, off_f, 0.f,
-                                         code_seed(p, i, 0)},
-                           EncSoA<D, St>{gout.base + i, (unsigned short*)(gout.base + p.N) + i, p.N, off_g, 0.f,
-                                         code_seed(p, i, 1)});
+        coded::rest_offsets<D, St>(p, s, dh, GFromArray{gr}, off_f, off_g);
+        coded::collide_outputs<D>(p, s, coded::DhArray{dh}, m, GFromArray{gr}, ph, pl,
+                                  EncSoA<D, St>{fout.base + i, (unsigned short*)(fout.base + p.N) + i, p.N, off_f, 0.f,
+                                                code_seed(p, i, 0)},
+                                  EncSoA<D, St>{gout.base + i, (unsigned short*)(gout.base + p.N) + i, p.N, off_g, 0.f,
+                                                code_seed(p, i, 1)});
     } else {
-        collide_outputs<D>(p, s, DhArray{dh}, m, GFromArray{gr}, nh[Q / 2], nl[Q / 2], SoAOut{fout.base + i, p.N},
-                           SoAOut{gout.base + i, p.N});
+        const SoAOut fo{fout.base + i, p.N}, go{gout.base + i, p.N};
+        stencil_from_nb<D>(nh, nl, grad, lap);
+        FlowMoments m;
+        flow_moments<D>(m, fr);
+        CellState s;
+        Residual R;
+        if constexpr (!PR) {
+            if (p.flags & kFlagDivU) {  // the w cs2 rho div(u) term of Xi (Sec. 2.3)
+                flow_closure<D, true>(p, ph, grad, lap, m, s, inv_rho, nu, div_stored<D>(p, us_in, x, y, z));
+                flow_relax<D>(m, s, inv_rho, nu, R);
+                for (int k = 0; k < D; ++k) us_out[k * p.N + i] = s.u[k];
+                collide_outputs<D, false, true>(p, s, R, m, GFromArray{gr}, ph, pl, fo, go);
+                return;
+            }
+        }
+        flow_closure<D>(p, ph, grad, lap, m, s, inv_rho, nu);
+        flow_relax<D>(m, s, inv_rho, nu, R);
+        if constexpr (PR)
+            collide_outputs<D, true>(p, s, R, m, GFromArray{gr}, ph, pl, fo, go, PhiUStep<D>{p, phiu, i});
+        else
+            collide_outputs<D>(p, s, R, m, GFromArray{gr}, ph, pl, fo, go);
     }
 }
 

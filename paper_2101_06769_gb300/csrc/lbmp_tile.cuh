@@ -25,26 +25,9 @@ namespace LBMP_TILE_NS {
 #ifndef LBMP_FUSED_MINB
 #define LBMP_FUSED_MINB 3
 #endif
-// 1: f' of the plane is staged by cp.async into shared memory with the g
-// copies (frees the registers of 27 loads in flight); 0: loaded to registers
-#ifndef LBMP_FUSED_FSMEM
-#define LBMP_FUSED_FSMEM 0
-#endif
-// 1: the 27 post-collision moment differences are parked in shared memory
-// between the collision set-up and the output loop
-#ifndef LBMP_FUSED_DHSMEM
-#define LBMP_FUSED_DHSMEM 1
-#endif
 // 1: the phase field on the reduced lattice D3Q7 (LBMP_FLAG_PHASE_REDUCED)
 #ifndef LBMP_PHASE_REDUCED
 #define LBMP_PHASE_REDUCED 0
-#endif
-// 1 (full phase lattice only): the phase-field outputs are emitted first, so
-// the staged pre-collision g of the plane is consumed before the flow
-// relaxation, which then parks its 27 moment differences in that g column
-// (no separate shared-memory array for them)
-#ifndef LBMP_FUSED_SPLIT
-#define LBMP_FUSED_SPLIT 0
 #endif
 // 1: the ring cells' g are loaded to registers and summed at once by the
 // ring threads (no shared-memory ring buffer)
@@ -72,13 +55,9 @@ constexpr int NRING = 2 * RX + 2 * TY;
 constexpr int Q3 = 27;
 constexpr bool PR = LBMP_PHASE_REDUCED != 0;
 constexpr int QG = PhaseLat<3, PR>::Q;  // phase-field populations
-constexpr bool kSplit = LBMP_FUSED_SPLIT != 0 && !PR;
 constexpr bool kRingReg = LBMP_FUSED_RINGREG != 0;
-constexpr bool kDhSmem = LBMP_FUSED_DHSMEM != 0 && !kSplit;
 constexpr size_t kSmemBytes =
-    sizeof(float) * ((2 * QG + (LBMP_FUSED_FSMEM + (kDhSmem ? 1 : 0)) * Q3) * NT + (kRingReg ? 0 : QG * NRING) +
-                     (PR ? 2 * 3 * NT : 0)) +
-    sizeof(float2) * 3 * PLANE;
+    sizeof(float) * (2 * QG * NT + (kRingReg ? 0 : QG * NRING) + (PR ? 2 * 3 * NT : 0)) + sizeof(float2) * 2 * PLANE;
 static_assert(NRING <= NT, "one thread per ring cell");
 
 __device__ __forceinline__ void cp_async4(float* smem, const float* gmem)
