@@ -116,7 +116,9 @@ void fill_devparams(lbmp_handle* h)
     q.neg_inv_tau = -q.inv_tau_phi;
     q.lam_sharp = (float)(d.lambda_phi * 4.0 / d.W);
     q.lam_n = (float)(d.tau_phi * d.lambda_phi * 4.0 / d.W);
-    q.lam_corr = (float)(d.tau_phi * d.lambda_phi * ((h->reduced && h->D == 3) ? 4.0 : 3.0));
+    const double ics2g = (h->reduced && h->D == 3) ? 4.0 : 3.0;
+    q.lam_corr = (float)(d.lambda_phi * ics2g);
+    q.lam_cn = (float)(d.tau_phi * d.lambda_phi * ics2g);
     q.g_accel = (float)d.g_accel;
     q.force_x = (float)d.force_x;
     const bool uniform = (h->params.flags & LBMP_FLAG_UNIFORM_FORCE) != 0;

@@ -28,7 +28,7 @@
 #endif
 #include <stdint.h>
 
-#include "lbmp_coded.cuh"
+#include "lbmp_repro.cuh"
 #include "lbmp_internal.h"
 #include "lbmp_tile.cuh"
 
@@ -319,14 +319,14 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
             Unroll<Q3>::run(CodeLoad<false>{Dp.fin, own, P, q});
         S.finish(z + 1, gS + (cur ^ 1) * Q3 * NT, phiS + sN * PLANE);
         if (ghost_plane(p, z + 1)) S.copy_phi(phiS + sC * PLANE, phiS + sN * PLANE);
-        coded::FlowMoments m;
+        repro::FlowMoments m;
         {
             float fr[Q3];
             if (P.lo || P.hi)
                 S.template decode_f<true>(z, P.lo, P.hi, q, fr);
             else
                 S.template decode_f<false>(z, false, false, q, fr);
-            coded::flow_moments<3>(m, fr);
+            repro::flow_moments<3>(m, fr);
         }
         __syncthreads();
         if (valid) {
@@ -340,8 +340,8 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
                 nl[a] = v.y;
             }
             float grad[3], lap;
-            coded::stencil_from_nb<3>(nh, nl, grad, lap);
-            coded::CellState s;
+            repro::stencil_from_nb<3>(nh, nl, grad, lap);
+            repro::CellState s;
             const cell_off self = P.zs[1] + own.ys[1] + own.xs[1];
             float* gcol = gS + cur * Q3 * NT + tid;  // this cell's decoded pre-collision g
             const GFromStrided gin{gcol, NT};
@@ -349,19 +349,19 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
             // holds the moment differences for the f' outputs.  The rest
             // offsets of the encoders are those of rest_offsets.
             float inv_rho, nu;
-            coded::flow_closure<3>(p, nh[13], grad, lap, m, s, inv_rho, nu);
-            const float gd = coded::gamma_dev<3>(s, C3);
+            repro::flow_closure<3>(p, nh[13], grad, lap, m, s, inv_rho, nu);
+            const float gd = repro::gamma_dev<3>(s, C3);
             const float kS = St::S / wint<3>(C3);
-            const EncCell<St> go{Dp.gout, Dp.rgout, self, kS * coded::phase_post<3>(p, s, C3, gin(C3), gd), 0.f,
+            const EncCell<St> go{Dp.gout, Dp.rgout, self, kS * repro::phase_post<3>(p, s, C3, gin(C3), gd), 0.f,
                                  code_seed(p, elem_index(self), 1)};
-            coded::phase_outputs<3>(p, s, gin, nh[13], nl[13], go);
+            repro::phase_outputs<3>(p, s, gin, nh[13], nl[13], go);
             float dh[27];
-            coded::flow_relax<3>(m, s, inv_rho, nu, dh);
+            repro::flow_relax<3>(m, s, inv_rho, nu, dh);
 #pragma unroll
             for (int a = 0; a < Q3; ++a) gcol[a * NT] = dh[a];
-            const EncCell<St> fo{Dp.fout, Dp.rfout, self, kS * coded::flow_post<3>(s, dh, C3, gd), 0.f,
+            const EncCell<St> fo{Dp.fout, Dp.rfout, self, kS * repro::flow_post<3>(s, dh, C3, gd), 0.f,
                                  code_seed(p, elem_index(self), 0)};
-            coded::flow_outputs<3>(s, coded::DhStrided{gcol, NT}, m, fo);
+            repro::flow_outputs<3>(s, repro::DhStrided{gcol, NT}, m, fo);
         }
         __syncthreads();
         const int t = sP;

@@ -12,6 +12,7 @@
 // term, Sec. 2.2): 5 staged g values, and the stored previous phi u of the
 // staged row copied with them.
 #include "lbmp_internal.h"
+#include "lbmp_repro.cuh"
 
 namespace lbmp {
 
@@ -179,13 +180,16 @@ __device__ __forceinline__ void stage_row(const DevParams& p, const DirPtrs2& D,
     }
     cp_async_commit();
     cp_async_wait_all();
-    float hi, lo;
-    if (tid < 2) {
-        phi_sum_phase<2, PR>([&](int r) { return sbuf[r * 2 + tid]; }, hi, lo);
-        prow[tid == 0 ? 0 : RW - 1] = make_float2(hi, lo);
-    }
-    phi_sum_phase<2, PR>([&](int r) { return gbuf[r * TX2 + tid]; }, hi, lo);
-    prow[tid + 1] = make_float2(hi, lo);
+    const auto phi_of = [](const auto& get) {
+        float hi, lo;
+        if constexpr (SX)
+            repro::phi_sum_phase<2, PR>(get, hi, lo);
+        else
+            phi_sum_phase<2, PR>(get, hi, lo);
+        return make_float2(hi, lo);
+    };
+    if (tid < 2) prow[tid == 0 ? 0 : RW - 1] = phi_of([&](int r) { return sbuf[r * 2 + tid]; });
+    prow[tid + 1] = phi_of([&](int r) { return gbuf[r * TX2 + tid]; });
 }
 
 // rows [y0, y1) of the segment starting at x0.  One barrier per row: every
@@ -230,33 +234,43 @@ __device__ __forceinline__ void fused2_segment(const DevParams& p, const DirPtrs
         for (int a = 0; a < Q2; ++a) fr[a] = __ldg(pulled2<SX>(D.fin, a, own, R));
         stage_row<PR, SX>(p, D, own, side, tid, y + 1, gS + (cur ^ 1) * QG * TX2, sS, phiS + sN * RW, phiu,
                       uS + (cur ^ 1) * 2 * TX2);
-        FlowMoments m;
-        flow_moments<2>(m, fr);
-        __syncthreads();
-        if (valid) {
-            float nh[Q2], nl[Q2];
-#pragma unroll
-            for (int a = 0; a < Q2; ++a) {
-                const int cy = Lat<2>::cy(a);
-                const float2 v = phiS[(cy < 0 ? sP : (cy == 0 ? sC : sN)) * RW + tid + 1 + Lat<2>::cx(a)];
-                nh[a] = v.x;
-                nl[a] = v.y;
+        const off2 self = R.ys[1] + own.xs[1];
+        const GFromStrided gin{gS + cur * QG * TX2 + tid, TX2};  // this cell's staged pre-collision g
+        const Out2 fo{D.fout, self}, go{D.gout, self};
+        const float* prev = uS + cur * 2 * TX2 + tid;
+        const auto nb = [&](int a) {  // phi of the stencil's neighbour a
+            const int cy = Lat<2>::cy(a);
+            return phiS[(cy < 0 ? sP : (cy == 0 ? sC : sN)) * RW + tid + 1 + Lat<2>::cx(a)];
+        };
+        if constexpr (SX) {  // reproduced to the last bit (lbmp_repro.cuh)
+            repro::FlowMoments m;
+            repro::flow_moments<2>(m, fr);
+            __syncthreads();
+            if (valid) {
+                const float2 c = nb(4);
+                float grad[3], lap, inv_rho, nu, dh[27];
+                repro::stencil_from<2>(nb, c, grad, lap);
+                repro::CellState s;
+                repro::flow_closure<2>(p, c.x, grad, lap, m, s, inv_rho, nu);
+                repro::flow_relax<2>(m, s, inv_rho, nu, dh);
+                repro::collide_outputs<2, PR>(p, s, repro::DhArray{dh}, m, gin, c.x, c.y, fo, go,
+                                              repro::PhiUStaged<2>{p, phiu, elem2(self), prev, TX2});
             }
-            float grad[3], lap;
-            stencil_from_nb<2>(nh, nl, grad, lap);
-            CellState s;
-            float inv_rho, nu;
-            flow_closure<2>(p, nh[4], grad, lap, m, s, inv_rho, nu);
-            Residual Rs;
-            flow_relax<2>(m, s, inv_rho, nu, Rs);
-            const off2 self = R.ys[1] + own.xs[1];
-            if constexpr (PR)
-                collide_outputs<2, true>(p, s, Rs, m, GFromStrided{gS + cur * QG * TX2 + tid, TX2}, nh[4],
-                                         nl[4], Out2{D.fout, self}, Out2{D.gout, self},
-                                         PhiUStaged<2>{p, phiu, elem2(self), uS + cur * 2 * TX2 + tid, TX2});
-            else
-                collide_outputs<2>(p, s, Rs, m, GFromStrided{gS + cur * Q2 * TX2 + tid, TX2}, nh[4], nl[4],
-                                   Out2{D.fout, self}, Out2{D.gout, self});
+        } else {
+            FlowMoments m;
+            flow_moments<2>(m, fr);
+            __syncthreads();
+            if (valid) {
+                const float2 c = nb(4);
+                float grad[3], lap, inv_rho, nu;
+                stencil_from<2>(nb, grad, lap);
+                CellState s;
+                flow_closure<2>(p, c.x, grad, lap, m, s, inv_rho, nu);
+                Residual Rs;
+                flow_relax<2>(m, s, inv_rho, nu, Rs);
+                collide_outputs<2, PR>(p, s, Rs, m, gin, c.x, c.y, fo, go,
+                                       PhiUStaged<2>{p, phiu, elem2(self), prev, TX2});
+            }
         }
     }
     __syncthreads();

@@ -18,7 +18,7 @@
 // reference pair (lbmp_kernels.cu), in the same order.
 #include <type_traits>
 
-#include "lbmp_coded.cuh"
+#include "lbmp_repro.cuh"
 #include "lbmp_internal.h"
 
 namespace lbmp {
@@ -262,7 +262,7 @@ __device__ __forceinline__ void fused2s_segment(const DevParams& p, const DirPtr
         for (int a = 0; a < Q2; ++a)
             if (a != C2) q[a] = pulled_code(D.fin, a, C, bq[a]);
         stage_g(y + 1, gS + (cur ^ 1) * Q2 * TX2, sN, sC);
-        coded::FlowMoments m;
+        repro::FlowMoments m;
         {
             const float* R0 = RF + (y & (kRefRows - 1)) * RW + tid + 1;
             float fr[Q2];
@@ -276,7 +276,7 @@ __device__ __forceinline__ void fused2s_segment(const DevParams& p, const DirPtr
                     fr[a] = dec_value<2, St>(a, St::dec(q[a]), R);
                 }
             }
-            coded::flow_moments<2>(m, fr);
+            repro::flow_moments<2>(m, fr);
         }
         cp_async_wait_all();
         __syncthreads();
@@ -290,19 +290,19 @@ __device__ __forceinline__ void fused2s_segment(const DevParams& p, const DirPtr
                 nl[a] = v.y;
             }
             float grad[3], lap;
-            coded::stencil_from_nb<2>(nh, nl, grad, lap);
-            coded::CellState s;
+            repro::stencil_from_nb<2>(nh, nl, grad, lap);
+            repro::CellState s;
             float dh[27];
             float inv_rho, nu;
-            coded::flow_closure<2>(p, nh[C2], grad, lap, m, s, inv_rho, nu);
-            coded::flow_relax<2>(m, s, inv_rho, nu, dh);
+            repro::flow_closure<2>(p, nh[C2], grad, lap, m, s, inv_rho, nu);
+            repro::flow_relax<2>(m, s, inv_rho, nu, dh);
             const off2s self = C.ys[1] + C.xs[1];
             const GFromStrided gi{gS + cur * Q2 * TX2 + tid, TX2};
             float off_f, off_g;
-            coded::rest_offsets<2, St>(p, s, dh, gi, off_f, off_g);
+            repro::rest_offsets<2, St>(p, s, dh, gi, off_f, off_g);
             const EncCell2<St> fo{D.fout, D.rfout, self, off_f, 0.f, code_seed(p, elem2s(self), 0)};
             const EncCell2<St> go{D.gout, D.rgout, self, off_g, 0.f, code_seed(p, elem2s(self), 1)};
-            coded::collide_outputs<2>(p, s, coded::DhArray{dh}, m, gi, nh[C2], nl[C2], fo, go);
+            repro::collide_outputs<2>(p, s, repro::DhArray{dh}, m, gi, nh[C2], nl[C2], fo, go);
         }
     }
     __syncthreads();

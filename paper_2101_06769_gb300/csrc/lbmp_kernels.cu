@@ -7,7 +7,7 @@
 // opposite population of the cell itself (Sec. 3.2 boundary treatment).
 #include <math.h>
 
-#include "lbmp_coded.cuh"
+#include "lbmp_repro.cuh"
 #include "lbmp_internal.h"
 
 namespace lbmp {
@@ -40,13 +40,15 @@ __global__ void phi_pass_kernel(DevParams p, Pop<D, St> g, float* __restrict__ p
             },
             hi, lo);
     } else {
-        phi_sum_phase<D, PR>(
-            [&](int r) {
-                int slot;
-                const long long c = pull_src_g<D, PR>(p, r, x, y, z, i, slot);
-                return g.load(slot, c);
-            },
-            hi, lo);
+        const auto get = [&](int r) {
+            int slot;
+            const long long c = pull_src_g<D, PR>(p, r, x, y, z, i, slot);
+            return g.load(slot, c);
+        };
+        if (D == 2 && p.sym_x)
+            repro::phi_sum_phase<D, PR>(get, hi, lo);
+        else
+            phi_sum_phase<D, PR>(get, hi, lo);
     }
     phi[i] = hi;  // phi = sum_a g_a (Sec. 2.2), as hi + lo
     phi[p.N + i] = lo;
@@ -118,23 +120,29 @@ __global__ void __launch_bounds__(128) step_simple_kernel(DevParams p, Pop<D, St
     }
     const float ph = nh[Q / 2], pl = nl[Q / 2];
     float grad[3], lap, inv_rho, nu;
-    if constexpr (St::shifted) {
-        coded::stencil_from_nb<D>(nh, nl, grad, lap);
-        coded::FlowMoments m;
-        coded::flow_moments<D>(m, fr);
-        coded::CellState s;
+    // the steps reproduced to the last bit: shifted storage, a symmetry x axis
+    const auto step_repro = [&](auto fo, auto go) {
+        repro::stencil_from_nb<D>(nh, nl, grad, lap);
+        repro::FlowMoments m;
+        repro::flow_moments<D>(m, fr);
+        repro::CellState s;
         float dh[27];
-        coded::flow_closure<D>(p, ph, grad, lap, m, s, inv_rho, nu);
-        coded::flow_relax<D>(m, s, inv_rho, nu, dh);
-        float off_f, off_g;
-        coded::rest_offsets<D, St>(p, s, dh, GFromArray{gr}, off_f, off_g);
-        coded::collide_outputs<D>(p, s, coded::DhArray{dh}, m, GFromArray{gr}, ph, pl,
-                                  EncSoA<D, St>{fout.base + i, (unsigned short*)(fout.base + p.N) + i, p.N, off_f, 0.f,
-                                                code_seed(p, i, 0)},
-                                  EncSoA<D, St>{gout.base + i, (unsigned short*)(gout.base + p.N) + i, p.N, off_g, 0.f,
-                                                code_seed(p, i, 1)});
+        repro::flow_closure<D>(p, ph, grad, lap, m, s, inv_rho, nu);
+        repro::flow_relax<D>(m, s, inv_rho, nu, dh);
+        if constexpr (St::shifted) repro::rest_offsets<D, St>(p, s, dh, GFromArray{gr}, fo.off, go.off);
+        repro::collide_outputs<D, PR>(p, s, repro::DhArray{dh}, m, GFromArray{gr}, ph, pl, fo, go,
+                                      repro::PhiUStaged<D>{p, phiu, i, phiu + i, (int)p.N});
+    };
+    if constexpr (St::shifted) {
+        step_repro(EncSoA<D, St>{fout.base + i, (unsigned short*)(fout.base + p.N) + i, p.N, 0.f, 0.f,
+                                 code_seed(p, i, 0)},
+                   EncSoA<D, St>{gout.base + i, (unsigned short*)(gout.base + p.N) + i, p.N, 0.f, 0.f,
+                                 code_seed(p, i, 1)});
     } else {
         const SoAOut fo{fout.base + i, p.N}, go{gout.base + i, p.N};
+        if constexpr (D == 2) {
+            if (p.sym_x) return step_repro(fo, go);
+        }
         stencil_from_nb<D>(nh, nl, grad, lap);
         FlowMoments m;
         flow_moments<D>(m, fr);
@@ -588,7 +596,8 @@ cudaError_t launch_get_state(lbmp_handle* h, double* dev_f, double* dev_g)
 }
 
 // ---------------------------------------------------------- observables
-// rho, u and p_h = P + cs2 u.grad(rho)/2 of one cell, as in the step.
+// rho, u and p_h = P + cs2 u.grad(rho)/2 of one cell, by the arithmetic of
+// the domain's step.
 template <int D, class St>
 __device__ void cell_macro(const DevParams& p, const Pop<D, St>& f, const float* __restrict__ phi, int x, int y,
                            int z, long long i, float& rho, float u[3], float& ph, const float* __restrict__ ustore)
@@ -602,14 +611,24 @@ __device__ void cell_macro(const DevParams& p, const Pop<D, St>& f, const float*
         nl[a] = phi[p.N + j];
     }
     float grad[3], lap;
-    stencil_from_nb<D>(nh, nl, grad, lap);
     float fr[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) fr[a] = pulled_value<D, St>(p, f, a, x, y, z, i);
+    float inv_rho, nu;
+    if (St::shifted || (D == 2 && p.sym_x)) {
+        repro::stencil_from_nb<D>(nh, nl, grad, lap);
+        repro::FlowMoments m;
+        repro::flow_moments<D>(m, fr);
+        repro::CellState s;
+        rho = repro::flow_closure<D>(p, nh[Q / 2], grad, lap, m, s, inv_rho, nu);
+        for (int k = 0; k < 3; ++k) u[k] = s.u[k];
+        ph = s.ph;
+        return;
+    }
+    stencil_from_nb<D>(nh, nl, grad, lap);
     FlowMoments m;
     flow_moments<D>(m, fr);
     CellState s;
-    float inv_rho, nu;
     if (ustore)
         rho = flow_closure<D, true>(p, nh[Q / 2], grad, lap, m, s, inv_rho, nu, div_stored<D>(p, ustore, x, y, z));
     else

@@ -1,24 +1,64 @@
-// lbmp_coded.cuh -- the per-cell arithmetic of the steps on shifted 16-bit
-// storage.
+// lbmp_repro.cuh -- the per-cell arithmetic of the steps whose results must be
+// reproduced to the last bit: shifted 16-bit storage, and D2Q9 with a symmetry
+// x axis.
 //
-// The update is that of lbmp_common.cuh, in the form in which it was first
-// written: opposite pairs of directions as the lanes of the paired
-// arithmetic, post-collision central moments taken back to populations axis by
-// axis.  The FP32 steps have since moved to a form with fewer instructions,
-// which rounds differently in the last bit.  FP32 states do not notice, but a
-// 16-bit step rounds every output to a code by a threshold drawn per code, so
-// a last-bit change turns some codes over, the turned codes change the next
-// step's phi and reference values, and within 20 to 40 steps 40 % of the FP16
-// codes differ by an ulp (references by 3e-5 of their norm in FP16, 2e-4 in
-// BF16).  Those are equally good states, but stored 16-bit runs would no longer
-// be reproduced; so the 16-bit kernels and their reference pair keep these
+// The update is that of lbmp_common.cuh in the form in which it was first
+// written: opposite pairs of directions as the lanes of the paired arithmetic,
+// post-collision central moments taken back to populations axis by axis, the
+// stencil over all neighbours of a cell.  The other FP32 steps have moved to a
+// form with 30 % fewer instructions that rounds differently in the last bit
+// (and is no further from 64 bits); their runs stay within 1e-5 of the earlier
+// ones for as long as they were compared (80 steps).  Two kinds of run do not:
+//   * a 16-bit step rounds every output to a code by a threshold drawn per
+//     code, so a last-bit change turns some codes over, and these change the
+//     next step's phi and references: after 20 to 40 steps 40 % of the FP16
+//     codes differ by an ulp and the references by 3e-5 of their norm (BF16:
+//     2e-4);
+//   * the droplet impacts that the symmetry axis is for (density ratio 1000)
+//     amplify a last-bit change: 1e-5 after 21 steps, 1e-3 after 42, 4e-3 (of
+//     the largest population) after 80, about as far as both forms are from
+//     64 bits.
+// Those are equally good states, but stored runs would not be continued on the
+// same trajectory; so these kernels, and their reference pair, keep these
 // functions.
 #pragma once
 
 #include "lbmp_common.cuh"
 
 namespace lbmp {
-namespace coded {
+namespace repro {
+
+template <int D, class Get>
+__device__ __forceinline__ void phi_sum(const Get& get, float& hi, float& lo)
+{
+    constexpr int Q = Lat<D>::Q;
+    constexpr int C = Q / 2;
+    float2 h = f2(get(C), 0.f), l = f2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < C; ++k) {
+        const int a = by_weight<D>(k);
+        const float2 v = f2(get(a), get(Q - 1 - a));
+        const float2 s = add2(h, v);
+        l = add2(l, add2(v, neg2(add2(s, neg2(h)))));
+        h = s;
+    }
+    // join the lanes exactly, then renormalise (|lo| <= ulp(hi)/2)
+    const float t = h.x + h.y;
+    const float bb = t - h.x;
+    const float e = (h.x - (t - bb)) + (h.y - bb);
+    const float lsum = (l.x + l.y) + e;
+    hi = t + lsum;
+    lo = lsum - (hi - t);
+}
+
+template <int D, bool PR, class Get>
+__device__ __forceinline__ void phi_sum_phase(const Get& get, float& hi, float& lo)
+{
+    if constexpr (PR)
+        phi_sum_red<D>(get, hi, lo);
+    else
+        repro::phi_sum<D>(get, hi, lo);
+}
 
 // Isotropic differences (Sec. 2.2) from the Q neighbour values
 // phi(x + c_a) = nh[a] + nl[a]: grad_i = 3 sum w c_i phi(x+c),
@@ -393,69 +433,176 @@ __device__ __forceinline__ float2 pair_phase(const DevParams& p, const CellState
     return fma2(f2(ws, ws), mul2(pm1, f2(cn0, cn0)), fma2(itau, fma2(f2(s.phi, s.phi), wgd, neg2(gi)), gi));
 }
 
-// The moving outputs of one cell in two passes, phase field first (it needs
-// only the closure, so the flow relaxation comes after it); the encoder then
-// takes the cell's conserved total, P + u.G (flow) or the incoming sum (phase
-// field), in place of the rest value.
+// d/dt(phi u) for collide_outputs, with the previous value at prev[k * stride]
+// (staged, or the stored array itself)
+// (prev[k * stride]); the new value goes to the stored array
+template <int D>
+struct PhiUStaged {
+    const DevParams& p;
+    float* phiu;
+    long long i;
+    const float* prev;
+    int stride;
+    __device__ __forceinline__ void operator()(const CellState& s, float d[3]) const
+    {
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            const float v = s.phi * s.u[k];
+            d[k] = v - prev[k * stride];
+            phiu[k * p.N + i] = v;
+        }
+        if (D == 2) d[2] = 0.f;
+    }
+};
+// The rest populations from the conservation identities (see below): the
+// flow total P + u.G less the moving outputs fs,
+// the phase-field total (gsum_hi, gsum_lo) less the compensated moving
+// outputs (gs, gl); or a shifted encoder takes the totals themselves.
+template <class Out>
+__device__ __forceinline__ void flow_rest(const CellState& s, const FlowMoments& m, float2 fs, const Out& fout,
+                                          int C)
+{
+    if constexpr (Out::kTotal)
+        fout.finish(m.P, s.uG);
+    else
+        fout(C, (m.P + s.uG) - (fs.x + fs.y));
+}
+template <class Out>
+__device__ __forceinline__ void phase_rest(float gsum_hi, float gsum_lo, float2 gs, float2 gl, const Out& gout, int GC)
+{
+    if constexpr (Out::kTotal) {
+        gout.finish(gsum_hi, gsum_lo);
+    } else {
+        float t = gs.x + gs.y;  // combine the lanes exactly
+        const float bb = t - gs.x;
+        const float e = (gs.x - (t - bb)) + (gs.y - bb);
+        gout(GC, (gsum_hi - t) + (gsum_lo - (gl.x + gl.y + e)));
+    }
+}
+
+// The phase-field update on the reduced lattice: g* = g + (g_eq - g)/tau +
+// w c.(lambda 4 phi(1-phi)/W n + lambda/cs2 d/dt(phi u)) with the
+// first-order equilibrium g_eq = w phi (1 + c.u/cs2), the sharpening source
+// and the correction term (Sec. 2.2), lanes (r, opposite); the rest slot
+// from the conserved total.
+template <int D, class GSrc, class Out, class DPhiU>
+__device__ __forceinline__ void phase_outputs_reduced(const DevParams& p, const CellState& s, const GSrc& gin,
+                                                      float gsum_hi, float gsum_lo, const Out& gout,
+                                                      const DPhiU& dphiu_fn, float2 gs, float2 gl)
+{
+    constexpr int GC = PhaseLat<D, true>::C;
+    constexpr float ics = PhaseLat<D, true>::inv_cs2;
+    const float2 itau = f2(p.inv_tau_phi, p.inv_tau_phi);
+    const float2 pm1 = f2(1.f, -1.f);
+    float qv[3];
+    dphiu_fn(s, qv);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) qv[i] = fmaf(p.lam_corr, qv[i], s.sharp * s.n[i]);
+#pragma unroll
+    for (int r = 0; r < GC; ++r) {
+        const int a = PhaseLat<D, true>::full(r);
+        const int cx = Lat<D>::cx(a), cy = Lat<D>::cy(a), cz = Lat<D>::cz(a);
+        const float w = PhaseLat<D, true>::w(r);
+        const float cu = cx * s.u[0] + cy * s.u[1] + cz * s.u[2];
+        const float cq = cx * qv[0] + cy * qv[1] + cz * qv[2];
+        const float wphi = w * s.phi;
+        const float t = wphi * ics * cu;
+        const float2 geq = fma2(pm1, f2(t, t), f2(wphi, wphi));
+        const float2 gi = f2(gin(r), gin(2 * GC - r));
+        const float2 go = fma2(f2(w, w), mul2(pm1, f2(cq, cq)), fma2(itau, add2(geq, neg2(gi)), gi));
+        gout(r, go.x);
+        gout(2 * GC - r, go.y);
+        two_sum2(gs, gl, go);
+    }
+    phase_rest(gsum_hi, gsum_lo, gs, gl, gout, GC);
+}
+
+// PR: g on the reduced phase lattice (gin / gout index its slots), with
+// dphiu(s, d) giving d/dt(phi u) of the cell for the correction term.
+template <int D, bool PR = false, class GSrc, class Out, class DH, class DPhiU = NoPhiU>
+__device__ __forceinline__ void collide_outputs(const DevParams& p, const CellState& s, const DH& dh,
+                                                const FlowMoments& m, const GSrc& gin, float gsum_hi,
+                                                float gsum_lo, const Out& fout, const Out& gout,
+                                                const DPhiU& dphiu_fn = DPhiU{})
+{
+    static_assert(!(PR && Out::kTotal), "the reduced phase lattice is stored in FP32 only");
+    constexpr int Q = Lat<D>::Q;
+    constexpr int C = Q / 2;
+    const float m15uu = -1.5f * s.uu;
+    float2 fs = f2(0.f, 0.f), gs = f2(0.f, 0.f), gl = f2(0.f, 0.f);
+#pragma unroll
+    for (int a = 0; a < C; ++a) {
+        const int b = Q - 1 - a;
+        float2 gd, wgd;
+        pair_gamma<D>(s, a, m15uu, gd, wgd);
+        const float2 fo = pair_flow<D>(s, a, gd, wgd, f2(dh[a], dh[b]));
+        fout(a, fo.x);
+        fout(b, fo.y);
+        fs = add2(fs, fo);
+        if constexpr (!PR) {
+            const float2 go = pair_phase<D>(p, s, a, wgd, f2(gin(a), gin(b)));
+            gout(a, go.x);
+            gout(b, go.y);
+            two_sum2(gs, gl, go);
+        }
+    }
+    // target totals: P + u.G (flow) and the incoming sum (phase field); the
+    // rest populations take the difference (conservation identities above),
+    // or a shifted encoder takes the totals themselves
+    flow_rest(s, m, fs, fout, C);
+    if constexpr (PR)
+        phase_outputs_reduced<D>(p, s, gin, gsum_hi, gsum_lo, gout, dphiu_fn, gs, gl);
+    else
+        phase_rest(gsum_hi, gsum_lo, gs, gl, gout, C);
+}
+
+// The same outputs in two passes, phase field first: phase_outputs needs only
+// the closure (CellState without ew), so a kernel can run it before
+// flow_relax and reuse the staged pre-collision g for the moment
+// differences; flow_outputs then emits f'.  Each value is formed by the same
+// operations as in collide_outputs, and the rest populations accumulate the
+// moving ones in the same order, so the results are identical.
 template <int D, class GSrc, class Out>
 __device__ __forceinline__ void phase_outputs(const DevParams& p, const CellState& s, const GSrc& gin, float gsum_hi,
                                               float gsum_lo, const Out& gout)
 {
     constexpr int Q = Lat<D>::Q;
+    constexpr int C = Q / 2;
     const float m15uu = -1.5f * s.uu;
+    float2 gs = f2(0.f, 0.f), gl = f2(0.f, 0.f);
 #pragma unroll
-    for (int a = 0; a < Q / 2; ++a) {
+    for (int a = 0; a < C; ++a) {
         const int b = Q - 1 - a;
         float2 gd, wgd;
         pair_gamma<D>(s, a, m15uu, gd, wgd);
         const float2 go = pair_phase<D>(p, s, a, wgd, f2(gin(a), gin(b)));
         gout(a, go.x);
         gout(b, go.y);
+        two_sum2(gs, gl, go);
         out_pair_done();
     }
-    gout.finish(gsum_hi, gsum_lo);
+    phase_rest(gsum_hi, gsum_lo, gs, gl, gout, C);
 }
 template <int D, class Out, class DH>
 __device__ __forceinline__ void flow_outputs(const CellState& s, const DH& dh, const FlowMoments& m, const Out& fout)
 {
     constexpr int Q = Lat<D>::Q;
+    constexpr int C = Q / 2;
     const float m15uu = -1.5f * s.uu;
+    float2 fs = f2(0.f, 0.f);
 #pragma unroll
-    for (int a = 0; a < Q / 2; ++a) {
+    for (int a = 0; a < C; ++a) {
         const int b = Q - 1 - a;
         float2 gd, wgd;
         pair_gamma<D>(s, a, m15uu, gd, wgd);
         const float2 fo = pair_flow<D>(s, a, gd, wgd, f2(dh[a], dh[b]));
         fout(a, fo.x);
         fout(b, fo.y);
+        fs = add2(fs, fo);
         out_pair_done();
     }
-    fout.finish(m.P, s.uG);
+    flow_rest(s, m, fs, fout, C);
 }
 
-// both in one pass
-template <int D, class GSrc, class Out, class DH>
-__device__ __forceinline__ void collide_outputs(const DevParams& p, const CellState& s, const DH& dh,
-                                                const FlowMoments& m, const GSrc& gin, float gsum_hi,
-                                                float gsum_lo, const Out& fout, const Out& gout)
-{
-    constexpr int Q = Lat<D>::Q;
-    const float m15uu = -1.5f * s.uu;
-#pragma unroll
-    for (int a = 0; a < Q / 2; ++a) {
-        const int b = Q - 1 - a;
-        float2 gd, wgd;
-        pair_gamma<D>(s, a, m15uu, gd, wgd);
-        const float2 fo = pair_flow<D>(s, a, gd, wgd, f2(dh[a], dh[b]));
-        fout(a, fo.x);
-        fout(b, fo.y);
-        const float2 go = pair_phase<D>(p, s, a, wgd, f2(gin(a), gin(b)));
-        gout(a, go.x);
-        gout(b, go.y);
-    }
-    fout.finish(m.P, s.uG);
-    gout.finish(gsum_hi, gsum_lo);
-}
-
-}  // namespace coded
+}  // namespace repro
 }  // namespace lbmp
