@@ -67,11 +67,20 @@ struct BatchDomain {
 
 // Launch shape of a persistent fused kernel over `tiles` tiles marching
 // through `nmarch` planes (rows in 2-D): planes per work item and grid size,
-// from the handle's options or the defaults (enough items for three rounds of
-// the full-occupancy grid, at least 8 planes per item: each item stages two
-// planes more than it updates, so longer items win until the rounds get
-// coarse; on the 128x128x512 RT workload 32 planes per item at 4 CTAs per
-// SM measured 0.852 ms per step, 16 planes 0.893 ms).
+// from the handle's options or the defaults.
+//
+// Default planes per item.  Where 8 or more planes per item leave three rounds
+// of the full-occupancy grid, the largest power-of-two part of the domain that
+// does: each item stages two planes more than it updates, so longer items win
+// until the rounds get coarse (128x128x512 RT: 32 planes 0.730 ms per step,
+// 16 planes 0.731, 64 planes 0.757).  A smaller domain cannot fill three
+// rounds; there the time is about rounds x (planes + 1.5) x (0.7 + occupancy),
+// the stages of one item times a stage's latency, which grows with the number
+// of CTAs that share an SM, and the rule takes the planes that make it
+// smallest.  Measured in us per step, 8 planes -> the rule's choice: D2Q9
+// 64x256 8.6 -> 3.5 (1 row), 400x250 10.0 -> 6.4 (2), 1024x512 17.1 -> 15.2
+// (4), 2048x1024 65.4 -> 61.2 (16); D3Q27 32^3 18.7 -> 7.3 (1 plane), 48^3
+// 18.6 -> 14.5 (2), 64^3 31.4 -> 26.3 (4).
 struct LaunchShape {
     int chunk, nitems, grid;
 };
@@ -84,8 +93,22 @@ inline LaunchShape launch_shape(const lbmp_handle* h, int tiles, int nmarch, int
     if (h->opt_chunk > 0) {
         chunk = h->opt_chunk < nmarch ? h->opt_chunk : nmarch;
     } else {
+        const long long slots = (long long)per_sm * sms;
         chunk = nmarch;
-        while (chunk > 8 && (long long)tiles * ((nmarch + chunk - 1) / chunk) < 3LL * per_sm * sms) chunk /= 2;
+        while (chunk > 8 && (long long)tiles * ((nmarch + chunk - 1) / chunk) < 3 * slots) chunk /= 2;
+        if ((long long)tiles * ((nmarch + chunk - 1) / chunk) < 3 * slots) {
+            double best = 0.0;
+            const int top = nmarch < 64 ? nmarch : 64;
+            for (int c = top; c >= 1; --c) {
+                const long long items = (long long)tiles * ((nmarch + c - 1) / c);
+                const long long rounds = (items + slots - 1) / slots;
+                const double cost = (double)rounds * (c + 1.5) * (0.7 + (double)items / (double)(rounds * slots));
+                if (c == top || cost < best) {
+                    best = cost;
+                    chunk = c;
+                }
+            }
+        }
     }
     LaunchShape L;
     L.chunk = chunk;
