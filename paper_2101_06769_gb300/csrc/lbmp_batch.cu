@@ -52,6 +52,8 @@ enum Kind {
     kKinds = 10
 };
 constexpr int kLast3 = kF32x3R;  // the D3Q27 kinds are kF32x3 .. kLast3
+// resident CTAs per SM of each kind's kernel
+constexpr int kCtas[kKinds] = {4, 3, 3, 4, 8, 6, 6, 8, 7, 7};
 
 int kind_of(const lbmp_handle* h)
 {
@@ -71,8 +73,8 @@ struct lbmp_batch {
     bool own_stream;  // created here: the legacy default stream cannot be captured
     cudaStream_t side;               // second branch of a step (D2Q9 members)
     cudaEvent_t fork, join;
-    int tile, chunk;                 // D3Q27 tile shape (LBMP_OPT_TILE values), planes per item (0 = 16)
-    int device;
+    int tile, chunk;                 // D3Q27 tile shape (LBMP_OPT_TILE values), planes per item (0 = by rule)
+    int device, sms;
     std::vector<Member> members;
     lbmp::BatchDomain* d_table;       // device, kMaxMembers entries, grouped by kind
     std::vector<lbmp::BatchDomain> h_table;
@@ -177,7 +179,8 @@ cudaError_t capture(lbmp_batch* b, int steps, int phase, cudaGraphExec_t* out)
     }
     cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
     if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+    // node priorities: a replay otherwise runs every node at the priority of the stream it is launched into
+    if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, cudaGraphInstantiateFlagUseNodePriority);
     if (g) cudaGraphDestroy(g);
     return e;
 }
@@ -195,7 +198,19 @@ cudaError_t rebuild(lbmp_batch* b, bool graphs = true)
     const bool fp32_2d = kind == kF32x2 || kind == kF32x2R || kind == kF32x2S || kind == kF32x2RS;
     const int TX = fp32_2d ? lbmp::batch2_tile_x() : ops3_of(b, kind).tile_x;
     const int TY = D == 3 ? ops3_of(b, kind).tile_y : 1;
-    const int chunk = b->chunk > 0 ? b->chunk : 16;
+    int chunk = b->chunk;
+    if (chunk <= 0) {
+        // a kind's members share one launch: the rule takes them together,
+        // with the CTAs per SM its kernel reaches
+        std::vector<int> tiles, nmarch;
+        for (const Member& m : b->members) {
+            if (m.left <= 0 || kind_of(m.h) != kind) continue;
+            const lbmp_grid& g = m.h->grid;
+            tiles.push_back(((g.nx + TX - 1) / TX) * (D == 3 ? (g.ny + TY - 1) / TY : 1));
+            nmarch.push_back(D == 3 ? g.nz : g.ny);
+        }
+        chunk = lbmp::planes_per_item(tiles.data(), nmarch.data(), (int)tiles.size(), (long long)kCtas[kind] * b->sms);
+    }
     for (const Member& m : b->members) {
         if (m.left <= 0 || kind_of(m.h) != kind) continue;
         const lbmp_handle* h = m.h;
@@ -283,7 +298,13 @@ LBMP_API int lbmp_batch_create(size_t hbm_budget, void* cuda_stream, lbmp_batch*
         e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
         b->own_stream = e == cudaSuccess;
     }
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
+    // the D2Q9 members' branch goes first where both have CTAs to place: the
+    // D3Q27 kernels fill every slot of the GPU, and the few short 2-D items
+    // would otherwise start when those end
+    int least = 0, greatest = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->side, cudaStreamNonBlocking, greatest);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_table, sizeof(lbmp::BatchDomain) * kMaxMembers);

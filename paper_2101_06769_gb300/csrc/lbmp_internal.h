@@ -65,22 +65,48 @@ struct BatchDomain {
     int tiles_x, tiles_y, chunk, item_begin, items;
 };
 
+// Default planes (rows in 2-D) per work item of `n` domains stepped by one
+// launch, domain k with tiles[k] tiles marching through nmarch[k] planes, on
+// `slots` resident CTAs.  Where 8 or more planes per item leave 2.5 rounds
+// of the full grid, the largest power-of-two part of the longest domain that
+// does: each item stages two planes more than it updates, so longer items win
+// until the rounds get coarse (128x128x512 RT: 32 planes 0.730 ms per step,
+// 16 planes 0.731, 64 planes 0.757).  Smaller work cannot fill 2.5 rounds;
+// there the time is about rounds x (planes + 1.5) x (0.7 + occupancy), the
+// stages of one item times a stage's latency, which grows with the number of
+// CTAs that share an SM, and the rule takes the planes that make it smallest.
+// Measured in us per step, 8 planes -> the rule's choice: D2Q9 64x256
+// 8.6 -> 3.5 (1 row), 400x250 10.0 -> 6.4 (2), 1024x512 17.1 -> 15.2 (4),
+// 2048x1024 65.4 -> 61.2 (16); D3Q27 32^3 18.7 -> 7.3 (1 plane), 48^3
+// 18.6 -> 14.5 (2), 64^3 31.4 -> 26.3 (4).
+inline int planes_per_item(const int* tiles, const int* nmarch, int n, long long slots)
+{
+    int longest = 1;
+    for (int k = 0; k < n; ++k) longest = nmarch[k] > longest ? nmarch[k] : longest;
+    const auto items = [&](int c) {
+        long long t = 0;
+        for (int k = 0; k < n; ++k) t += (long long)tiles[k] * ((nmarch[k] + c - 1) / c);
+        return t;
+    };
+    int chunk = longest;
+    while (chunk > 8 && 2 * items(chunk) < 5 * slots) chunk /= 2;
+    if (2 * items(chunk) >= 5 * slots) return chunk;
+    const int top = longest < 64 ? longest : 64;
+    double best = 0.0;
+    for (int c = top; c >= 1; --c) {
+        const long long it = items(c), rounds = (it + slots - 1) / slots;
+        const double cost = (double)rounds * (c + 1.5) * (0.7 + (double)it / (double)(rounds * slots));
+        if (c == top || cost < best) {
+            best = cost;
+            chunk = c;
+        }
+    }
+    return chunk;
+}
+
 // Launch shape of a persistent fused kernel over `tiles` tiles marching
 // through `nmarch` planes (rows in 2-D): planes per work item and grid size,
 // from the handle's options or the defaults.
-//
-// Default planes per item.  Where 8 or more planes per item leave three rounds
-// of the full-occupancy grid, the largest power-of-two part of the domain that
-// does: each item stages two planes more than it updates, so longer items win
-// until the rounds get coarse (128x128x512 RT: 32 planes 0.730 ms per step,
-// 16 planes 0.731, 64 planes 0.757).  A smaller domain cannot fill three
-// rounds; there the time is about rounds x (planes + 1.5) x (0.7 + occupancy),
-// the stages of one item times a stage's latency, which grows with the number
-// of CTAs that share an SM, and the rule takes the planes that make it
-// smallest.  Measured in us per step, 8 planes -> the rule's choice: D2Q9
-// 64x256 8.6 -> 3.5 (1 row), 400x250 10.0 -> 6.4 (2), 1024x512 17.1 -> 15.2
-// (4), 2048x1024 65.4 -> 61.2 (16); D3Q27 32^3 18.7 -> 7.3 (1 plane), 48^3
-// 18.6 -> 14.5 (2), 64^3 31.4 -> 26.3 (4).
 struct LaunchShape {
     int chunk, nitems, grid;
 };
@@ -89,30 +115,12 @@ inline LaunchShape launch_shape(const lbmp_handle* h, int tiles, int nmarch, int
     if (per_sm < 1) per_sm = 1;
     const int ctas = (h->opt_ctas > 0 && h->opt_ctas < per_sm) ? h->opt_ctas : per_sm;
     const long long cap = (long long)ctas * sms;
-    int chunk;
-    if (h->opt_chunk > 0) {
-        chunk = h->opt_chunk < nmarch ? h->opt_chunk : nmarch;
-    } else {
-        const long long slots = (long long)per_sm * sms;
-        chunk = nmarch;
-        while (chunk > 8 && (long long)tiles * ((nmarch + chunk - 1) / chunk) < 3 * slots) chunk /= 2;
-        if ((long long)tiles * ((nmarch + chunk - 1) / chunk) < 3 * slots) {
-            double best = 0.0;
-            const int top = nmarch < 64 ? nmarch : 64;
-            for (int c = top; c >= 1; --c) {
-                const long long items = (long long)tiles * ((nmarch + c - 1) / c);
-                const long long rounds = (items + slots - 1) / slots;
-                const double cost = (double)rounds * (c + 1.5) * (0.7 + (double)items / (double)(rounds * slots));
-                if (c == top || cost < best) {
-                    best = cost;
-                    chunk = c;
-                }
-            }
-        }
-    }
     LaunchShape L;
-    L.chunk = chunk;
-    L.nitems = tiles * ((nmarch + chunk - 1) / chunk);
+    if (h->opt_chunk > 0)
+        L.chunk = h->opt_chunk < nmarch ? h->opt_chunk : nmarch;
+    else
+        L.chunk = planes_per_item(&tiles, &nmarch, 1, (long long)per_sm * sms);
+    L.nitems = tiles * ((nmarch + L.chunk - 1) / L.chunk);
     L.grid = (int)(L.nitems < cap ? L.nitems : cap);
     return L;
 }
