@@ -15,4 +15,6 @@
 #define LBMP_FUSED3_LAUNCH launch_step_fused3
 #define LBMP_BATCH3_OPS batch3_ops_32x4
 #define LBMP_FUSED3_WITH_COMMON 1
+#define LBMP_FUSED3_OBS 1
+#define LBMP_FUSED3_OBS_LAUNCH launch_obs_fused3
 #include "lbmp_fused3_body.cuh"

@@ -31,10 +31,16 @@
 // LBMP_BATCH3_OPS (the name of its batch-kernel table) and, for a tile shape
 // other than the default, LBMP_FUSED_TX / _TY and LBMP_TILE_NS;
 // LBMP_FUSED3_WITH_COMMON adds the pieces shared by every tile shape.
+// LBMP_FUSED3_OBS = 1 adds the observables' kernel and its launcher
+// LBMP_FUSED3_OBS_LAUNCH.
 // LBMP_PHASE_REDUCED = 1 builds the kernel for the reduced phase lattice
 // (D3Q7 g with the first-order equilibrium and the correction term, Sec. 2.2;
 // the stored previous phi u is read and replaced per cell).
 #pragma once
+
+#ifndef LBMP_FUSED3_OBS
+#define LBMP_FUSED3_OBS 0
+#endif
 
 #include <string.h>
 
@@ -280,6 +286,97 @@ __global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_batchg3_kernel(const
     }
 }
 
+#if LBMP_FUSED3_OBS
+// The observables of the current state in the same march, without outputs:
+// phi of a plane from register loads of the own and ring cells' g, the stencil
+// by layers, f' and the closure; the running sums stay in registers.  Reads
+// each population once and stores no phi array, where a phi pass and a pass of
+// 27-neighbour gathers over its (hi, lo) arrays read 2.3 times the bytes and
+// spent most of their time on index divisions and FP64 instructions: 1.92 ->
+// 0.444 ms on 128x128x512, 1.81 GB read at 4.1 TB/s (5 CTAs per SM, with
+// spills: 0.475).  Grid-strided work items, partial sums per CTA in
+// a fixed order (deterministic).  cols: phi on the spike column (nx/2, ny/2)
+// and the bubble column (0, 0), or null.
+__device__ __forceinline__ void obs_phi(const DevParams& p, const DirPtrs& D, const Column& own, const Column& ring,
+                                        const ThreadGeo& T, int zz, float2* slot)
+{
+    Plane P;
+    set_plane(P, p, plane_src(p, zz));
+    if (P.lo || P.hi) {
+        ring_phi_direct<true>(D, own, P, slot + T.oslot);
+        if (T.tid < NRING) ring_phi_direct<true>(D, ring, P, slot + T.rslot);
+    } else {
+        ring_phi_direct<false>(D, own, P, slot + T.oslot);
+        if (T.tid < NRING) ring_phi_direct<false>(D, ring, P, slot + T.rslot);
+    }
+}
+
+__global__ void __launch_bounds__(NT, 4) obs_fused3_kernel(DevParams p, FusedArgs A, DirPtrs Dp,
+                                                           double* __restrict__ part, double* __restrict__ cols)
+{
+    __shared__ float2 phiS[2 * PLANE];
+    __shared__ double sm[4 * (NT / 32)];
+    const ThreadGeo T = thread_geo();
+    const float2* cell = phiS + T.oslot;
+    const auto layer = [&](int slot, LayerSums& L) {
+        layer_sums<3>([&](int dx, int dy) { return cell[slot * PLANE + dy * RX + dx]; }, L);
+    };
+    ObsAcc acc = {};
+    for (int item = blockIdx.x; item < A.nitems; item += gridDim.x) {
+        const int tile = item % (A.tiles_x * A.tiles_y);
+        const int z0 = (item / (A.tiles_x * A.tiles_y)) * A.chunk, z1 = min(z0 + A.chunk, p.nz);
+        const int x0 = (tile % A.tiles_x) * TX, y0 = (tile / A.tiles_x) * TY;
+        const int x = x0 + T.tx, y = y0 + T.ty;
+        Column own, ring;
+        set_column(own, p, pmod(x, p.nx), pmod(y, p.ny));
+        set_column(ring, p, pmod(x0 + T.lx, p.nx), pmod(y0 + T.ly, p.ny));
+        const bool valid = x < p.nx && y < p.ny;
+        const int col = cols && valid ? ((x == p.nx / 2 && y == p.ny / 2) ? 1 : 0) + ((x == 0 && y == 0) ? 2 : 0) : 0;
+        obs_phi(p, Dp, own, ring, T, z0 - 1, phiS);
+        obs_phi(p, Dp, own, ring, T, z0, phiS + PLANE);
+        LayerSums below, here;
+        __syncthreads();
+        layer(0, below);
+        layer(1, here);
+        __syncthreads();
+        for (int z = z0; z < z1; ++z) {
+            const int cur = (z - z0) & 1;
+            Plane P;
+            set_plane(P, p, z);
+            FlowMoments m;
+            {
+                float fr[Q3];
+                if (P.lo || P.hi)
+                    Unroll<Q3>::run(PullLoad<true>{Dp.fin, own, P, fr});
+                else
+                    Unroll<Q3>::run(PullLoad<false>{Dp.fin, own, P, fr});
+                flow_moments<3>(m, fr);
+            }
+            obs_phi(p, Dp, own, ring, T, z + 1, phiS + cur * PLANE);
+            __syncthreads();
+            LayerSums above;
+            layer(cur, above);
+            if (valid) {
+                float grad[3], lap, inv_rho, nu;
+                stencil_from_layers<3>(below, here, above, grad, lap);
+                CellState s;
+                const float rho = flow_closure<3>(p, here.c.x, grad, lap, m, s, inv_rho, nu);
+                obs_cell(acc, here.c, rho, s.u, s.ph);
+                if (col) {
+                    const double v = (double)here.c.x + (double)here.c.y;
+                    if (col & 1) cols[z] = v;
+                    if (col & 2) cols[p.nz + z] = v;
+                }
+            }
+            below = here;
+            here = above;
+        }
+        __syncthreads();
+    }
+    obs_block(acc, sm, part + 4 * blockIdx.x);
+}
+#endif
+
 struct LaunchCfg {
     int device = -1;
     int per_sm = 0, sms = 0;
@@ -369,6 +466,54 @@ cudaError_t launch_batch_grid(const BatchDomain* host, const BatchDomain* dev, i
 
 }  // namespace
 
+namespace {
+DirPtrs dir_ptrs(const lbmp_handle* h)
+{
+    DirPtrs D;
+    const int s = h->parity, d = 1 - h->parity;
+    for (int a = 0; a < Q3; ++a) {
+        const size_t off = (size_t)a * (size_t)h->N;
+        D.fin[a] = h->f[s] + off;
+        D.fout[a] = h->f[d] + off;
+    }
+    for (int r = 0; r < QG; ++r) {
+        const size_t off = (size_t)r * (size_t)h->N;
+        D.gin[r] = h->g[s] + off;
+        D.gout[r] = h->g[d] + off;
+    }
+    return D;
+}
+}  // namespace
+
+#if LBMP_FUSED3_OBS
+cudaError_t LBMP_FUSED3_OBS_LAUNCH(lbmp_handle* h, double* part, int max_parts, int* nparts, double* cols)
+{
+    static LaunchCfg cfg;
+    if (cfg.device != h->device) {
+        int per_sm = 0, sms = 0;
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, obs_fused3_kernel, NT, 0);
+        if (e != cudaSuccess) return e;
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+        if (e != cudaSuccess) return e;
+        cfg.per_sm = per_sm > 0 ? per_sm : 1;
+        cfg.sms = sms;
+        cfg.device = h->device;
+    }
+    FusedArgs A;
+    A.phiu = nullptr;
+    A.tiles_x = (h->grid.nx + TX - 1) / TX;
+    A.tiles_y = (h->grid.ny + TY - 1) / TY;
+    const int tiles = A.tiles_x * A.tiles_y;
+    A.chunk = planes_per_item(&tiles, &h->grid.nz, 1, (long long)cfg.per_sm * cfg.sms);
+    A.nitems = tiles * ((h->grid.nz + A.chunk - 1) / A.chunk);
+    int grid = A.nitems < cfg.per_sm * cfg.sms ? A.nitems : cfg.per_sm * cfg.sms;
+    if (grid > max_parts) grid = max_parts;
+    *nparts = grid;
+    obs_fused3_kernel<<<grid, NT, 0, h->stream>>>(h->dp, A, dir_ptrs(h), part, cols);
+    return cudaGetLastError();
+}
+#endif
+
 const Batch3Ops LBMP_BATCH3_OPS = {TX, TY, prepare_batch, nullptr, launch_batch_grid, kGridMembers};
 
 cudaError_t LBMP_FUSED3_LAUNCH(lbmp_handle* h)
@@ -386,18 +531,7 @@ cudaError_t LBMP_FUSED3_LAUNCH(lbmp_handle* h)
         g_cfg.sms = sms;
         g_cfg.device = h->device;
     }
-    DirPtrs D;
-    const int s = h->parity, d = 1 - h->parity;
-    for (int a = 0; a < Q3; ++a) {
-        const size_t off = (size_t)a * (size_t)h->N;
-        D.fin[a] = h->f[s] + off;
-        D.fout[a] = h->f[d] + off;
-    }
-    for (int r = 0; r < QG; ++r) {
-        const size_t off = (size_t)r * (size_t)h->N;
-        D.gin[r] = h->g[s] + off;
-        D.gout[r] = h->g[d] + off;
-    }
+    const DirPtrs D = dir_ptrs(h);
     FusedArgs A;
     A.phiu = h->phiu;
     A.tiles_x = (h->grid.nx + TX - 1) / TX;

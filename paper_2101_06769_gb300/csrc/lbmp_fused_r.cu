@@ -11,4 +11,6 @@
 #define LBMP_FUSED3_LAUNCH launch_step_fused3_red
 #define LBMP_BATCH3_OPS batch3_ops_red
 #define LBMP_FUSED3_WITH_COMMON 0
+#define LBMP_FUSED3_OBS 1
+#define LBMP_FUSED3_OBS_LAUNCH launch_obs_fused3_red
 #include "lbmp_fused3_body.cuh"

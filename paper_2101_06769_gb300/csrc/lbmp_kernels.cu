@@ -642,8 +642,8 @@ template <int D, class St>
 __global__ void __launch_bounds__(256) obs_partial_kernel(DevParams p, Pop<D, St> f, const float* __restrict__ phi,
                                                           double* __restrict__ part, const float* __restrict__ ustore)
 {
-    __shared__ double sm[4][256];
-    double mass = 0.0, ke = 0.0, um = 0.0, bad = 0.0;
+    __shared__ double sm[4 * 8];
+    ObsAcc acc = {};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.N;
          i += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
@@ -651,32 +651,9 @@ __global__ void __launch_bounds__(256) obs_partial_kernel(DevParams p, Pop<D, St
         if (D == 3 && (z < p.zb || z >= p.ze)) continue;  // a z-slab's ghost planes belong to its neighbours
         float rho, u[3], ph;
         cell_macro<D, St>(p, f, phi, x, y, z, i, rho, u, ph, ustore);
-        const double uu = (double)u[0] * u[0] + (double)u[1] * u[1] + (double)u[2] * u[2];
-        const double ph_i = (double)phi[i] + (double)phi[p.N + i];
-        mass += ph_i;
-        ke += 0.5 * rho * uu;
-        const double un = sqrt(uu);
-        if (!(un <= um)) um = un;
-        if (!isfinite(ph_i) || !isfinite(uu) || !isfinite(ph)) bad += 1.0;
+        obs_cell(acc, f2(phi[i], phi[p.N + i]), rho, u, ph);
     }
-    const int t = threadIdx.x;
-    sm[0][t] = mass;
-    sm[1][t] = ke;
-    sm[2][t] = um;
-    sm[3][t] = bad;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (t < s) {
-            sm[0][t] += sm[0][t + s];
-            sm[1][t] += sm[1][t + s];
-            const double o = sm[2][t + s];
-            if (!(o <= sm[2][t])) sm[2][t] = o;
-            sm[3][t] += sm[3][t + s];
-        }
-        __syncthreads();
-    }
-    if (t == 0)
-        for (int k = 0; k < 4; ++k) part[4 * blockIdx.x + k] = sm[k][0];
+    obs_block(acc, sm, part + 4 * blockIdx.x);
 }
 
 // fixed-order final reduction of the partials (deterministic for a fixed grid)
@@ -744,6 +721,67 @@ __global__ void probe_kernel(DevParams p, Pop<D, St> f, const float* __restrict_
     }
 }
 
+// The probes of a domain without a phi array (FP32 D3Q27, two sets): the block
+// forms phi (hi, lo) of the 5^3 cells around its probe from g, then p_h of the
+// inner 27 as probe_kernel does.
+template <bool PR>
+__global__ void __launch_bounds__(128) probe_pull_kernel(DevParams p, Pop<3, StoreF32> f, Pop<3, StoreF32> g, int px,
+                                                         int py, int pz, double* __restrict__ out)
+{
+    __shared__ float2 ps[125];
+    __shared__ double sm[27];
+    const int t = threadIdx.x;
+    const bool first = blockIdx.x == 0;  // probe (px, py, pz), then the origin
+    const int cx = first ? px : 0, cy = first ? py : 0, cz = first ? pz : 0;
+    // an offset of up to two cells in a domain of at least two: wrapped until inside
+    const auto wrap = [](int v, int n) {
+        const int r = v % n;
+        return r < 0 ? r + n : r;
+    };
+    const auto vert = [&](int z) { return p.vert_periodic ? wrap(z, p.nz) : (z < 0 ? 0 : (z >= p.nz ? p.nz - 1 : z)); };
+    if (t < 125) {
+        const int x = wrap(cx + t % 5 - 2, p.nx), y = wrap(cy + (t / 5) % 5 - 2, p.ny), z = vert(cz + t / 25 - 2);
+        const long long i = ((long long)z * p.ny + y) * p.nx + x;
+        float hi, lo;
+        phi_sum_phase<3, PR>(
+            [&](int r) {
+                int slot;
+                const long long c = pull_src_g<3, PR>(p, r, x, y, z, i, slot);
+                return g.load(slot, c);
+            },
+            hi, lo);
+        ps[t] = f2(hi, lo);
+    }
+    __syncthreads();
+    if (t < 27) {
+        const int dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = t / 9 - 1;
+        // beyond a wall the probe's block takes the wall cell itself, whose
+        // stencil lies around that cell
+        const int zt = vert(cz + dz), oz = p.vert_periodic ? dz : zt - cz;
+        const int x = wrap(cx + dx, p.nx), y = wrap(cy + dy, p.ny);
+        const long long i = ((long long)zt * p.ny + y) * p.nx + x;
+        float grad[3], lap, fr[27], inv_rho, nu;
+        stencil_from<3>(
+            [&](int a) {
+                return ps[(dx + Lat<3>::cx(a) + 2) + 5 * (dy + Lat<3>::cy(a) + 2) + 25 * (oz + Lat<3>::cz(a) + 2)];
+            },
+            grad, lap);
+#pragma unroll
+        for (int a = 0; a < 27; ++a) fr[a] = pulled_value<3, StoreF32>(p, f, a, x, y, zt, i);
+        FlowMoments m;
+        flow_moments<3>(m, fr);
+        CellState s;
+        flow_closure<3>(p, ps[(dx + 2) + 5 * (dy + 2) + 25 * (oz + 2)].x, grad, lap, m, s, inv_rho, nu);
+        sm[t] = s.ph;
+    }
+    __syncthreads();
+    if (t == 0) {
+        double v = 0.0;
+        for (int k = 0; k < 27; ++k) v += sm[k];
+        out[blockIdx.x] = v / 27;
+    }
+}
+
 // phi on the spike column (nx/2, ny/2) and the bubble column (0, 0)
 template <int D>
 __global__ void column_kernel(DevParams p, const float* __restrict__ phi, double* __restrict__ out)
@@ -786,8 +824,37 @@ struct ObsL {
     }
 };
 
+// FP32 D3Q27 domains on two population sets: one march, no phi array.  The
+// variants with a phi array of their own (divergence term, in-place storage),
+// z-slabs (whose ghost planes hold no complete g) and the other lattices and
+// storage forms run the phi pass and the gathers.
+static bool obs_marches(const lbmp_handle* h)
+{
+    return h->D == 3 && h->params.storage == LBMP_FP32 && !h->divu && !h->aa && !h->slab;
+}
+
+static cudaError_t obs_march(lbmp_handle* h, double* out, bool full)
+{
+    int nparts = 0;
+    double* cols = full ? out + 16 : nullptr;
+    cudaError_t e = h->reduced ? launch_obs_fused3_red(h, h->red, h->red_blocks, &nparts, cols)
+                               : launch_obs_fused3(h, h->red, h->red_blocks, &nparts, cols);
+    if (e != cudaSuccess) return e;
+    obs_final_kernel<<<1, 256, 0, h->stream>>>(h->red, nparts, out);
+    if (full) {
+        const Pop<3, StoreF32> f = pop_of<3, StoreF32>(h, h->f[h->parity]), g = pop_of<3, StoreF32>(h, h->g[h->parity]);
+        const int* pr = h->probe;
+        if (h->reduced)
+            probe_pull_kernel<true><<<2, 128, 0, h->stream>>>(h->dp, f, g, pr[0], pr[1], pr[2], out + 4);
+        else
+            probe_pull_kernel<false><<<2, 128, 0, h->stream>>>(h->dp, f, g, pr[0], pr[1], pr[2], out + 4);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_observables(lbmp_handle* h, double* dev_out)
 {
+    if (obs_marches(h)) return obs_march(h, dev_out, true);
     cudaError_t e = launch_phi_pass(h);
     if (e != cudaSuccess) return e;
     return dispatch(h, ObsL{h, dev_out, true});
@@ -795,6 +862,7 @@ cudaError_t launch_observables(lbmp_handle* h, double* dev_out)
 
 cudaError_t launch_mass(lbmp_handle* h, double* dev_out4)
 {
+    if (obs_marches(h)) return obs_march(h, dev_out4, false);
     cudaError_t e = launch_phi_pass(h);
     if (e != cudaSuccess) return e;
     return dispatch(h, ObsL{h, dev_out4, false});
