@@ -11,17 +11,19 @@
 //     rotation, one new plane per step: g over the tile plus two rings (a ring
 //     cell's phi pulls from one cell further out), f' over the tile plus one
 //     ring.  Offsets of the staged plane cells are computed once per segment.
-//   * cp.async has no 2-byte form, so a g code is copied as the aligned
-//     32-bit word that holds it.  nx is even and tile origins are multiples
-//     of TX, so the half a thread needs is fixed by its lane parity and the
-//     direction's cx (the cell itself for a bounced population), and one byte
-//     permute extracts it.
-//   * f' codes are loaded to registers (2-byte loads) and decoded after the
-//     reference planes are in place.
+//   * the 16-bit codes of the own and ring cells' g(z+1) and of f'(z) are loaded
+//     to registers (2-byte loads) and decoded when the reference planes are in
+//     place; the own cells' decoded g is kept in shared memory for the collision
+//     one plane later.
 //   * the ghost plane beyond a wall (mirrored phi, reading A17) is a copy of
 //     the wall plane's phi instead of a second staging of that plane.
-// the output pair loops keep their memory operations in order (lower register footprint)
-#define LBMP_OUT_ORDERED 1
+// What bounds it: instruction issue (every value is decoded and encoded; DRAM
+// stands at a fifth of its rate) and the instruction cache.  It issues
+// 3045 instructions per cell (3553 when g codes were staged as 32-bit words and
+// the two population sets were emitted in two passes): 1.10 ms per step on the
+// 128x128x512 RT workload in FP16 (1.21 before), BF16 1.08 (1.18).  With the
+// ring's codes loaded beside the others (400 B of spills) 1.22, at four CTAs
+// per SM (500 B of spills) 1.12.
 #define LBMP_TILE_NS tile16
 #ifndef LBMP_FUSED_BYTEOFF
 #define LBMP_FUSED_BYTEOFF 2
@@ -38,8 +40,8 @@ namespace {
 
 using namespace LBMP_TILE_NS;
 
-// the encoder of one cell's outputs (as EncPtr) at a cell offset of the tile
-// geometry: the codes at base + offset, the reference at its 4-byte slot
+// the encoder of one cell's outputs at a cell offset of the tile geometry: the
+// codes at base + offset, the reference at its 4-byte slot
 template <class St>
 struct EncCell {
     static constexpr bool kTotal = true;
@@ -49,12 +51,12 @@ struct EncCell {
     float off;
     mutable float sq;
     unsigned seed;  // code_seed of the writer cell (stochastic rounding)
-    __device__ __forceinline__ void operator()(int a, float v) const
+    __device__ __forceinline__ void pair(int a, float2 v) const
     {
-        const float W = wint<3>(a);
-        const unsigned short c = enc_code<St>(fmaf(v, St::S / W, -off), seed, a);
-        *at_cell(qb[a], self) = c;
-        sq += St::dec(c) * (W * St::s);
+        unsigned short ca, cb;
+        encode_pair<3, St>(a, v, off, seed, sq, ca, cb);
+        *at_cell(qb[a], self) = ca;
+        *at_cell(qb[26 - a], self) = cb;
     }
     __device__ __forceinline__ void finish(float th, float tl) const
     {
@@ -64,9 +66,7 @@ struct EncCell {
 
 constexpr int C3 = 13;
 constexpr int GX = TX + 4, GY = TY + 4, GPLANE = GX * GY;  // g reference plane: tile + two rings
-// the moment differences are parked in the consumed g column: no array of their own
-constexpr size_t kSmem16 = sizeof(float2) * 3 * PLANE +
-                           sizeof(float) * (2 * Q3 * NT + Q3 * NRING + 4 * GPLANE + 4 * PLANE) +
+constexpr size_t kSmem16 = sizeof(float2) * 3 * PLANE + sizeof(float) * (2 * Q3 * NT + 4 * GPLANE + 4 * PLANE) +
                            sizeof(int) * (GPLANE + PLANE);
 
 struct DirPtrs16 {
@@ -104,24 +104,6 @@ __device__ __forceinline__ void load_ref_plane(const DevParams& p, const float* 
     for (int e = tid; e < size; e += NT) cp_async4(d + e, base + off[e]);
 }
 
-// aligned 32-bit word holding the code of the pulled g population a
-template <bool Walls>
-struct StageWord {
-    const DirPtrs16& D;
-    const Column& C;
-    const Plane& P;
-    float* buf;
-    int stride;
-    template <int a>
-    __device__ __forceinline__ void step() const
-    {
-        if constexpr (a != C3) {
-            const unsigned short* src = pulled<Walls, a>(D.gin, C, P);
-            cp_async4(buf + a * stride, (const float*)((uintptr_t)src & ~(uintptr_t)3));
-        }
-    }
-};
-
 template <bool Walls>
 struct CodeLoad {
     const unsigned short* const* base;
@@ -135,39 +117,59 @@ struct CodeLoad {
     }
 };
 
-// Decode the staged words of one cell and sum phi (hi, lo) from the exact
-// parts of the values (phi_sum_shifted); Keep: also store the decoded values
-// in place (the tile's own cells, whose values the collision reads; ring
-// cells need phi only).  R0 is
-// the reference plane of the staged plane, Rm / Rp the planes below / above;
-// slot is the cell's index in the reference-plane layout of row length RL;
-// selA / selB pick the half of a word for a source of the cell's own / the
-// other x parity.
-template <bool Walls, class St, bool Keep>
-__device__ __forceinline__ void decode_g(const float* Rm, const float* R0, const float* Rp, int slot, int RL,
-                                         unsigned selA, unsigned selB, bool lo, bool hi, float* buf, int stride,
-                                         float& phi_hi, float& phi_lo)
+// pulled codes of one cell to registers
+__device__ __forceinline__ void load_codes(const unsigned short* const* base, const Column& C, const Plane& P_,
+                                           unsigned short* q)
 {
+    if (P_.lo || P_.hi)  // uniform across the CTA
+        Unroll<Q3>::run(CodeLoad<true>{base, C, P_, q});
+    else
+        Unroll<Q3>::run(CodeLoad<false>{base, C, P_, q});
+}
+
+// references of the writers of the pulled pair (a, opp(a)): slot is the cell's
+// index in the reference-plane layout of row length RL, Rm / R0 / Rp the
+// planes below, at and above the cell
+template <bool Walls>
+__device__ __forceinline__ float2 pair_refs(int a, const float* Rm, const float* R0, const float* Rp, int slot, int RL,
+                                            bool lo, bool hi)
+{
+    const int cx = Lat<3>::cx(a), cy = Lat<3>::cy(a), cz = Lat<3>::cz(a);
+    const auto ref = [&](int sx, int sy, int sz) {  // writer x - (sx, sy, sz)
+        if (Walls && ((sz == 1 && lo) || (sz == -1 && hi))) return R0[slot];
+        return (sz == 1 ? Rm : (sz == -1 ? Rp : R0))[slot - sx - sy * RL];
+    };
+    return f2(ref(cx, cy, cz), ref(-cx, -cy, -cz));
+}
+
+// Decode the codes q of one cell's g and sum phi (hi, lo) from the exact
+// parts of the values (phi_sum_shifted); Keep: also store the decoded values
+// at buf[a * stride] (the tile's own cells, whose values the collision reads;
+// ring cells need phi only).
+template <bool Walls, class St, bool Keep>
+__device__ __forceinline__ float2 decode_g(const unsigned short* q, const float* Rm, const float* R0, const float* Rp,
+                                           int slot, bool lo, bool hi, float* buf, int stride)
+{
+    float2 phi;
     phi_sum_shifted<3>(
-        [&](int a, float& wr, float& wq) {
-            const int cx = Lat<3>::cx(a), cy = Lat<3>::cy(a), cz = Lat<3>::cz(a);
-            const float W = wint<3>(a);
-            if (a == C3) {
-                wr = W * R0[slot];
-                wq = 0.f;
-                if (Keep) buf[a * stride] = wr;
-            } else {
-                const bool bounced = Walls && ((cz == 1 && lo) || (cz == -1 && hi));
-                const float* Rpl = cz == 1 ? Rm : (cz == -1 ? Rp : R0);
-                const float R = bounced ? R0[slot] : Rpl[slot - cx - cy * RL];
-                const unsigned sel = (cx == 0 || bounced) ? selA : selB;
-                const float qv = St::dec_word(__float_as_uint(buf[a * stride]), sel);
-                wr = W * R;
-                wq = qv * (W * St::s);
-                if (Keep) buf[a * stride] = dec_value<3, St>(a, qv, R);  // = wr + wq, rounded once
+        [&]() {
+            const float v = wint<3>(C3) * R0[slot];
+            if (Keep) buf[C3 * stride] = v;
+            return v;
+        },
+        [&](int a, float2& wr, float2& wq) {
+            const int b = Q3 - 1 - a;
+            const float2 R = pair_refs<Walls>(a, Rm, R0, Rp, slot, GX, lo, hi);
+            const float2 qv = f2(St::dec(q[a]), St::dec(q[b]));
+            decode_pair<3, St>(a, R, qv, wr, wq);
+            if (Keep) {
+                const float2 v = decode_pair<3, St>(a, R, qv);  // = wr + wq, rounded once
+                buf[a * stride] = v.x;
+                buf[b * stride] = v.y;
             }
         },
-        phi_hi, phi_lo);
+        phi.x, phi.y);
+    return phi;
 }
 
 template <class St>
@@ -177,65 +179,57 @@ struct Seg16 {
     const ThreadGeo& T;
     const Column& own;
     const Column& ring;
-    float* rS;
     float* RG;
     float* RF;
     const int* offG;
     const int* offF;
 
-    // copies for plane zz: reference planes zz+2 (g) and zz+1 (f'), and the
-    // g code words of the tile and ring cells (unless zz is a ghost plane)
-    __device__ __forceinline__ void issue(int zz, float* gbuf) const
+    // reference planes zz+2 (g) and zz+1 (f') into their rotation slots
+    __device__ __forceinline__ void issue_refs(int zz) const
     {
-        const int tid = T.tid;
-        load_ref_plane(p, D.rgin, zz + 2, RG, GPLANE, offG, tid);
-        load_ref_plane(p, D.rfin, zz + 1, RF, PLANE, offF, tid);
-        if (!ghost_plane(p, zz)) {
-            Plane P;
-            set_plane(P, p, plane_src(p, zz));
-            if (P.lo || P.hi) {  // uniform across the CTA
-                Unroll<Q3>::run(StageWord<true>{D, own, P, gbuf + tid, NT});
-                if (tid < NRING) Unroll<Q3>::run(StageWord<true>{D, ring, P, rS + tid, NRING});
-            } else {
-                Unroll<Q3>::run(StageWord<false>{D, own, P, gbuf + tid, NT});
-                if (tid < NRING) Unroll<Q3>::run(StageWord<false>{D, ring, P, rS + tid, NRING});
-            }
-        }
+        load_ref_plane(p, D.rgin, zz + 2, RG, GPLANE, offG, T.tid);
+        load_ref_plane(p, D.rfin, zz + 1, RF, PLANE, offF, T.tid);
         cp_async_commit();
     }
 
-    // wait for the copies; decode plane zz (unless a ghost) and write its phi
-    __device__ __forceinline__ void finish(int zz, float* gbuf, float2* phi_plane) const
+    // codes of plane zz of the own cell
+    __device__ __forceinline__ void load_g(int zz, unsigned short* qo) const
     {
-        cp_async_wait_all();
         if (ghost_plane(p, zz)) return;
-        const int pz = plane_src(p, zz);
-        const bool lo = !p.vert_periodic && pz == 0, hi = !p.vert_periodic && pz == p.nz - 1;
+        Plane P;
+        set_plane(P, p, plane_src(p, zz));
+        load_codes(D.gin, own, P, qo);
+    }
+
+    // decode plane zz (unless a ghost) and write its phi; the ring cells' codes
+    // are loaded here (with the own and f' codes they would spill)
+    template <bool Walls>
+    __device__ __forceinline__ void phi_of(int zz, bool lo, bool hi, const unsigned short* qo, float* gbuf,
+                                           float2* phi_plane) const
+    {
         const float* Rm = RG + ((zz + 7) & 3) * GPLANE;
         const float* R0 = RG + ((zz + 8) & 3) * GPLANE;
         const float* Rp = RG + ((zz + 9) & 3) * GPLANE;
-        const int tid = T.tid;
-        const unsigned oA = (T.tx & 1) ? St::kSelHi : St::kSelLo, oB = (T.tx & 1) ? St::kSelLo : St::kSelHi;
-        const int ogs = (T.ty + 2) * GX + T.tx + 2;
-        float h, l;
-        if (lo || hi) {
-            if (tid < NRING) {
-                const unsigned rA = (T.lx & 1) ? St::kSelHi : St::kSelLo, rB = (T.lx & 1) ? St::kSelLo : St::kSelHi;
-                decode_g<true, St, false>(Rm, R0, Rp, (T.ly + 2) * GX + T.lx + 2, GX, rA, rB, lo, hi, rS + tid, NRING, h,
-                                          l);
-                phi_plane[T.rslot] = make_float2(h, l);
-            }
-            decode_g<true, St, true>(Rm, R0, Rp, ogs, GX, oA, oB, lo, hi, gbuf + tid, NT, h, l);
-        } else {
-            if (tid < NRING) {
-                const unsigned rA = (T.lx & 1) ? St::kSelHi : St::kSelLo, rB = (T.lx & 1) ? St::kSelLo : St::kSelHi;
-                decode_g<false, St, false>(Rm, R0, Rp, (T.ly + 2) * GX + T.lx + 2, GX, rA, rB, false, false,
-                                           rS + tid, NRING, h, l);
-                phi_plane[T.rslot] = make_float2(h, l);
-            }
-            decode_g<false, St, true>(Rm, R0, Rp, ogs, GX, oA, oB, false, false, gbuf + tid, NT, h, l);
+        if (T.tid < NRING) {
+            Plane P;
+            set_plane(P, p, plane_src(p, zz));
+            unsigned short qr[Q3];
+            load_codes(D.gin, ring, P, qr);
+            phi_plane[T.rslot] =
+                decode_g<Walls, St, false>(qr, Rm, R0, Rp, (T.ly + 2) * GX + T.lx + 2, lo, hi, nullptr, 0);
         }
-        phi_plane[T.oslot] = make_float2(h, l);
+        phi_plane[T.oslot] =
+            decode_g<Walls, St, true>(qo, Rm, R0, Rp, (T.ty + 2) * GX + T.tx + 2, lo, hi, gbuf + T.tid, NT);
+    }
+    __device__ __forceinline__ void finish(int zz, const unsigned short* qo, float* gbuf, float2* phi_plane) const
+    {
+        if (ghost_plane(p, zz)) return;
+        const int pz = plane_src(p, zz);
+        const bool lo = !p.vert_periodic && pz == 0, hi = !p.vert_periodic && pz == p.nz - 1;
+        if (lo || hi)
+            phi_of<true>(zz, lo, hi, qo, gbuf, phi_plane);
+        else
+            phi_of<false>(zz, false, false, qo, gbuf, phi_plane);
     }
 
     // phi of the ghost plane = phi of the wall plane (each thread copies the
@@ -253,18 +247,14 @@ struct Seg16 {
         const float* Rm = RF + ((z + 7) & 3) * PLANE;
         const float* R0 = RF + ((z + 8) & 3) * PLANE;
         const float* Rp = RF + ((z + 9) & 3) * PLANE;
-        const int o = T.oslot;
+        fr[C3] = wint<3>(C3) * R0[T.oslot];
 #pragma unroll
-        for (int a = 0; a < Q3; ++a) {
-            const int cx = Lat<3>::cx(a), cy = Lat<3>::cy(a), cz = Lat<3>::cz(a);
-            if (a == C3) {
-                fr[a] = wint<3>(C3) * R0[o];
-            } else {
-                const bool bounced = Walls && ((cz == 1 && lo) || (cz == -1 && hi));
-                const float* Rpl = cz == 1 ? Rm : (cz == -1 ? Rp : R0);
-                const float R = bounced ? R0[o] : Rpl[o - cx - cy * RX];
-                fr[a] = dec_value<3, St>(a, St::dec(q[a]), R);
-            }
+        for (int a = 0; a < C3; ++a) {
+            const int b = Q3 - 1 - a;
+            const float2 R = pair_refs<Walls>(a, Rm, R0, Rp, T.oslot, RX, lo, hi);
+            const float2 v = decode_pair<3, St>(a, R, f2(St::dec(q[a]), St::dec(q[b])));
+            fr[a] = v.x;
+            fr[b] = v.y;
         }
     }
 };
@@ -274,9 +264,8 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
                                                 float* smem, int x0, int y0, int z0, int z1)
 {
     float2* phiS = (float2*)smem;                // (hi, lo) [3][PLANE]
-    float* gS = (float*)(phiS + 3 * PLANE);      // [2][27][NT] staged words, decoded in place
-    float* rS = gS + 2 * Q3 * NT;                // [27][NRING] ring cells
-    float* RG = rS + Q3 * NRING;                 // [4][GPLANE] g references
+    float* gS = (float*)(phiS + 3 * PLANE);      // [2][27][NT] decoded own g
+    float* RG = gS + 2 * Q3 * NT;                // [4][GPLANE] g references
     float* RF = RG + 4 * GPLANE;                 // [4][PLANE] f' references
     int* offG = (int*)(RF + 4 * PLANE);
     int* offF = offG + GPLANE;
@@ -289,38 +278,39 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
         offG[e] = pmod(y0 + e / GX - 2, p.ny) * p.nx + pmod(x0 + e % GX - 2, p.nx);
     for (int e = tid; e < PLANE; e += NT) offF[e] = pmod(y0 + e / RX - 1, p.ny) * p.nx + pmod(x0 + e % RX - 1, p.nx);
     __syncthreads();
-    const Seg16<St> S{p, Dp, T, own, ring, rS, RG, RF, offG, offF};
+    const Seg16<St> S{p, Dp, T, own, ring, RG, RF, offG, offF};
+    unsigned short qo[Q3];
     // reference planes needed before the first two stagings
     load_ref_plane(p, Dp.rgin, z0 - 2, RG, GPLANE, offG, tid);
     load_ref_plane(p, Dp.rgin, z0 - 1, RG, GPLANE, offG, tid);
     load_ref_plane(p, Dp.rgin, z0, RG, GPLANE, offG, tid);
     load_ref_plane(p, Dp.rfin, z0 - 1, RF, PLANE, offF, tid);
-    cp_async_commit();
-    cp_async_wait_all();
-    __syncthreads();
     int sP = 0, sC = 1, sN = 2;
-    S.issue(z0 - 1, gS + Q3 * NT);
-    S.finish(z0 - 1, gS + Q3 * NT, phiS + sP * PLANE);
-    __syncthreads();
-    S.issue(z0, gS);
-    S.finish(z0, gS, phiS + sC * PLANE);
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {  // planes z0 - 1 and z0
+        S.load_g(z0 - 1 + k, qo);
+        cp_async_commit();
+        cp_async_wait_all();
+        __syncthreads();
+        S.finish(z0 - 1 + k, qo, gS + (k ^ 1) * Q3 * NT, phiS + (k ? sC : sP) * PLANE);
+        S.issue_refs(z0 - 1 + k);
+    }
+    cp_async_wait_all();
     if (ghost_plane(p, z0 - 1)) S.copy_phi(phiS + sC * PLANE, phiS + sP * PLANE);
     __syncthreads();
     for (int z = z0; z < z1; ++z) {
         const int cur = (z - z0) & 1;
-        // g(z+1) words and the next reference planes in flight while the f'(z) codes load
-        S.issue(z + 1, gS + (cur ^ 1) * Q3 * NT);
+        // the codes of g(z+1) and f'(z) and the next reference planes in flight together
+        S.issue_refs(z + 1);
+        S.load_g(z + 1, qo);
         Plane P;
         set_plane(P, p, z);
-        unsigned short q[Q3];
-        if (P.lo || P.hi)
-            Unroll<Q3>::run(CodeLoad<true>{Dp.fin, own, P, q});
-        else
-            Unroll<Q3>::run(CodeLoad<false>{Dp.fin, own, P, q});
-        S.finish(z + 1, gS + (cur ^ 1) * Q3 * NT, phiS + sN * PLANE);
-        if (ghost_plane(p, z + 1)) S.copy_phi(phiS + sC * PLANE, phiS + sN * PLANE);
         repro::FlowMoments m;
         {
+            unsigned short q[Q3];
+            load_codes(Dp.fin, own, P, q);
+            S.finish(z + 1, qo, gS + (cur ^ 1) * Q3 * NT, phiS + sN * PLANE);
+            if (ghost_plane(p, z + 1)) S.copy_phi(phiS + sC * PLANE, phiS + sN * PLANE);
             float fr[Q3];
             if (P.lo || P.hi)
                 S.template decode_f<true>(z, P.lo, P.hi, q, fr);
@@ -328,40 +318,31 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
                 S.template decode_f<false>(z, false, false, q, fr);
             repro::flow_moments<3>(m, fr);
         }
+        cp_async_wait_all();
         __syncthreads();
         if (valid) {
-            float nh[Q3], nl[Q3];
-#pragma unroll
-            for (int a = 0; a < Q3; ++a) {
-                const int cz = Lat<3>::cz(a);
-                const float2* pl = phiS + (cz < 0 ? sP : (cz == 0 ? sC : sN)) * PLANE;
-                const float2 v = pl[T.oslot + Lat<3>::cy(a) * RX + Lat<3>::cx(a)];
-                nh[a] = v.x;
-                nl[a] = v.y;
-            }
-            float grad[3], lap;
-            repro::stencil_from_nb<3>(nh, nl, grad, lap);
+            const float2* pm = phiS + sP * PLANE + T.oslot;
+            const float2* pc = phiS + sC * PLANE + T.oslot;
+            const float2* pn = phiS + sN * PLANE + T.oslot;
+            const float2 centre = pc[0];
+            float grad[3], lap, inv_rho, nu, dh[27];
+            repro::stencil_from<3>(
+                [&](int a) {
+                    const int cz = Lat<3>::cz(a);
+                    return (cz < 0 ? pm : (cz == 0 ? pc : pn))[Lat<3>::cy(a) * RX + Lat<3>::cx(a)];
+                },
+                centre, grad, lap);
             repro::CellState s;
-            const cell_off self = P.zs[1] + own.ys[1] + own.xs[1];
-            float* gcol = gS + cur * Q3 * NT + tid;  // this cell's decoded pre-collision g
-            const GFromStrided gin{gcol, NT};
-            // g first (it needs only the closure); its decoded column then
-            // holds the moment differences for the f' outputs.  The rest
-            // offsets of the encoders are those of rest_offsets.
-            float inv_rho, nu;
-            repro::flow_closure<3>(p, nh[13], grad, lap, m, s, inv_rho, nu);
-            const float gd = repro::gamma_dev<3>(s, C3);
-            const float kS = St::S / wint<3>(C3);
-            const EncCell<St> go{Dp.gout, Dp.rgout, self, kS * repro::phase_post<3>(p, s, C3, gin(C3), gd), 0.f,
-                                 code_seed(p, elem_index(self), 1)};
-            repro::phase_outputs<3>(p, s, gin, nh[13], nl[13], go);
-            float dh[27];
+            repro::flow_closure<3>(p, centre.x, grad, lap, m, s, inv_rho, nu);
             repro::flow_relax<3>(m, s, inv_rho, nu, dh);
-#pragma unroll
-            for (int a = 0; a < Q3; ++a) gcol[a * NT] = dh[a];
-            const EncCell<St> fo{Dp.fout, Dp.rfout, self, kS * repro::flow_post<3>(s, dh, C3, gd), 0.f,
-                                 code_seed(p, elem_index(self), 0)};
-            repro::flow_outputs<3>(s, repro::DhStrided{gcol, NT}, m, fo);
+            const cell_off self = P.zs[1] + own.ys[1] + own.xs[1];
+            const GFromStrided gin{gS + cur * Q3 * NT + tid, NT};  // this cell's decoded pre-collision g
+            float off_f, off_g;
+            repro::rest_offsets<3, St>(p, s, dh, gin, off_f, off_g);
+            repro::collide_outputs<3>(
+                p, s, repro::DhArray{dh}, m, gin, centre.x, centre.y,
+                EncCell<St>{Dp.fout, Dp.rfout, self, off_f, 0.f, code_seed(p, elem_index(self), 0)},
+                EncCell<St>{Dp.gout, Dp.rgout, self, off_g, 0.f, code_seed(p, elem_index(self), 1)});
         }
         __syncthreads();
         const int t = sP;

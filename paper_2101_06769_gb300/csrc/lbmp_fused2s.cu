@@ -126,8 +126,8 @@ __device__ __forceinline__ void set_cell2(Cell2& C, const DevParams& p, int x, i
     C.ys[2] = (off2s)((y == 0 ? p.ny - 1 : y - 1) * p.nx) * kUnit2s;
 }
 
-// the encoder of one cell's outputs (as EncPtr) at a cell offset: the codes
-// at base + offset, the reference at its 4-byte slot
+// the encoder of one cell's outputs at a cell offset: the codes at base +
+// offset, the reference at its 4-byte slot
 template <class St>
 struct EncCell2 {
     static constexpr bool kTotal = true;
@@ -137,12 +137,12 @@ struct EncCell2 {
     float off;
     mutable float sq;
     unsigned seed;  // code_seed of the writer cell (stochastic rounding)
-    __device__ __forceinline__ void operator()(int a, float v) const
+    __device__ __forceinline__ void pair(int a, float2 v) const
     {
-        const float W = wint<2>(a);
-        const unsigned short c = enc_code<St>(fmaf(v, St::S / W, -off), seed, a);
-        *at2s(qb[a], self) = c;
-        sq += St::dec(c) * (W * St::s);
+        unsigned short ca, cb;
+        encode_pair<2, St>(a, v, off, seed, sq, ca, cb);
+        *at2s(qb[a], self) = ca;
+        *at2s(qb[8 - a], self) = cb;
     }
     __device__ __forceinline__ void finish(float th, float tl) const
     {
@@ -175,24 +175,29 @@ __device__ __forceinline__ float2 decode_g_cell(const DevParams& p, const DirPtr
     Cell2 C;
     set_cell2(C, p, x, pmod(yy, p.ny));
     const float* R0 = RG + (yy & (kRefRows - 1)) * GW + e;
+    const auto code_and_ref = [&](int a, float& c, float& r) {
+        bool bounced;
+        const int cx = Lat<2>::cx(a), cy = Lat<2>::cy(a);
+        c = St::dec(pulled_code(D.gin, a, C, bounced));
+        r = bounced ? R0[0] : RG[((yy - cy) & (kRefRows - 1)) * GW + e - cx];
+    };
     float hi, lo;
     phi_sum_shifted<2>(
-        [&](int a, float& wr, float& wq) {
-            const float W = wint<2>(a);
-            if (a == C2) {
-                wr = W * R0[0];
-                wq = 0.f;
-                if (Keep) buf[a * TX2] = wr;
-                return;
+        [&]() {
+            const float v = wint<2>(C2) * R0[0];
+            if (Keep) buf[C2 * TX2] = v;
+            return v;
+        },
+        [&](int a, float2& wr, float2& wq) {
+            float2 q, R;
+            code_and_ref(a, q.x, R.x);
+            code_and_ref(Q2 - 1 - a, q.y, R.y);
+            decode_pair<2, St>(a, R, q, wr, wq);
+            if (Keep) {
+                const float2 v = decode_pair<2, St>(a, R, q);
+                buf[a * TX2] = v.x;
+                buf[(Q2 - 1 - a) * TX2] = v.y;
             }
-            bool bounced;
-            const unsigned short c = pulled_code(D.gin, a, C, bounced);
-            const int cx = Lat<2>::cx(a), cy = Lat<2>::cy(a);
-            const float R = bounced ? R0[0] : RG[((yy - cy) & (kRefRows - 1)) * GW + e - cx];
-            const float qv = St::dec(c);
-            wr = W * R;
-            wq = qv * (W * St::s);
-            if (Keep) buf[a * TX2] = dec_value<2, St>(a, qv, R);
         },
         hi, lo);
     return make_float2(hi, lo);

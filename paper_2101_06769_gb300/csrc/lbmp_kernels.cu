@@ -32,11 +32,20 @@ __global__ void phi_pass_kernel(DevParams p, Pop<D, St> g, float* __restrict__ p
     cell_xyz(p, i, x, y, z);
     float hi, lo;
     if constexpr (St::shifted) {
+        const auto parts = [&](int a, float& wr, float& wq) {
+            int dir;
+            const long long c = pull_src<D>(p, a, x, y, z, i, dir);
+            g.load_parts(dir, c, wr, wq);
+        };
         phi_sum_shifted<D>(
-            [&](int a, float& wr, float& wq) {
-                int dir;
-                const long long c = pull_src<D>(p, a, x, y, z, i, dir);
-                g.load_parts(dir, c, wr, wq);
+            [&]() {
+                float wr, wq;
+                parts(Lat<D>::Q / 2, wr, wq);
+                return wr;
+            },
+            [&](int a, float2& wr, float2& wq) {
+                parts(a, wr.x, wq.x);
+                parts(Lat<D>::Q - 1 - a, wr.y, wq.y);
             },
             hi, lo);
     } else {

@@ -71,16 +71,14 @@ __device__ __forceinline__ void stencil_from(const NB& nb, float2 centre, float 
 {
     constexpr int Q = Lat<D>::Q;
     constexpr int C = Q / 2;
-    const float2 hc = f2(-centre.x, -centre.x), lc = f2(-centre.y, -centre.y);
     float gx = 0.f, gy = 0.f, gz = 0.f;
     float2 ls = f2(0.f, 0.f);
 #pragma unroll
     for (int a = 0; a < C; ++a) {
         const int b = Q - 1 - a;
         const float w = Lat<D>::w(a);
-        const float2 va = nb(a), vb = nb(b);
         // phi(x + c) - phi(x) and phi(x - c) - phi(x), hi and lo parts differenced first
-        const float2 dd = add2(add2(f2(va.x, vb.x), hc), add2(f2(va.y, vb.y), lc));
+        const float2 dd = f2(pair_diff(nb(a), centre), pair_diff(nb(b), centre));
         ls = fma2(f2(w, w), dd, ls);
         const float d = w * (dd.x - dd.y);
         if (Lat<D>::cx(a)) gx += Lat<D>::cx(a) * d;
@@ -179,14 +177,14 @@ __device__ __forceinline__ float flow_closure(const DevParams& p, float phi, con
     for (int i = 0; i < 3; ++i) {
         s.u[i] = (D == 2 && i == 2) ? 0.f : (3.0f * m.J[i] + 0.5f * F[i]) * inv_rho;
         s.n[i] = (D == 2 && i == 2) ? 0.f : grad[i] * inv_g;
-        s.G[i] = (D == 2 && i == 2) ? 0.f : p.drho * grad[i] / 3.0f;
+        s.G[i] = (D == 2 && i == 2) ? 0.f : third(__fmul_rn(p.drho, grad[i]));
         s.F[i] = F[i];
     }
     const float ux = s.u[0], uy = s.u[1], uz = s.u[2];
     s.uG = ux * s.G[0] + uy * s.G[1] + uz * s.G[2];
     s.uF = ux * F[0] + uy * F[1] + uz * F[2];
     s.uu = ux * ux + uy * uy + uz * uz;
-    s.rcs2 = rho / 3.0f;
+    s.rcs2 = third(rho);
     s.ph = m.P + 0.5f * s.uG;
     s.phi = phi;
     s.sharp = p.lam_sharp * phi * (1.0f - phi);
@@ -259,16 +257,27 @@ __device__ __forceinline__ void flow_relax(const FlowMoments& m, CellState& s, f
     // Kronecker inverse about u: per axis (k0,k1,k2) -> (c=-1, 0, +1)
     // m1 = k1 + u k0, m2 = k2 + 2u k1 + u^2 k0; f(0) = k0 - m2, f(+-1) = (m2 +- m1)/2
     constexpr int NZ = (D == 3) ? 3 : 1;
+    // (along x first: a line holds k2 alone, k1 alone, or k0 and k2)
 #pragma unroll
     for (int ic = 0; ic < NZ; ++ic)
 #pragma unroll
         for (int ib = 0; ib < 3; ++ib) {
             const int o = 3 * ib + 9 * ic;
-            const float k0 = k[o], k1 = k[o + 1], k2 = k[o + 2];
-            const float m1 = k1 + ux * k0, m2 = k2 + 2.f * ux * k1 + ux * ux * k0;
-            k[o] = 0.5f * (m2 - m1);
-            k[o + 1] = k0 - m2;
-            k[o + 2] = 0.5f * (m2 + m1);
+            if (ib == 0 && ic == 0) {
+                const float k2 = k[o + 2];
+                k[o] = k[o + 2] = 0.5f * k2;
+                k[o + 1] = -k2;
+            } else if (((ib + ic) & 1) != 0) {
+                const float m1 = k[o + 1], m2 = __fmul_rn(2.f * ux, m1);
+                k[o] = 0.5f * (m2 - m1);
+                k[o + 1] = -m2;
+                k[o + 2] = 0.5f * (m2 + m1);
+            } else {
+                const float k0 = k[o], m1 = __fmul_rn(ux, k0), m2 = fmaf(__fmul_rn(ux, ux), k0, k[o + 2]);
+                k[o] = 0.5f * (m2 - m1);
+                k[o + 1] = k0 - m2;
+                k[o + 2] = 0.5f * (m2 + m1);
+            }
         }
 #pragma unroll
     for (int ic = 0; ic < NZ; ++ic)
@@ -536,15 +545,14 @@ __device__ __forceinline__ void collide_outputs(const DevParams& p, const CellSt
         float2 gd, wgd;
         pair_gamma<D>(s, a, m15uu, gd, wgd);
         const float2 fo = pair_flow<D>(s, a, gd, wgd, f2(dh[a], dh[b]));
-        fout(a, fo.x);
-        fout(b, fo.y);
+        out_pair<Q>(fout, a, fo);
         fs = add2(fs, fo);
         if constexpr (!PR) {
             const float2 go = pair_phase<D>(p, s, a, wgd, f2(gin(a), gin(b)));
-            gout(a, go.x);
-            gout(b, go.y);
+            out_pair<Q>(gout, a, go);
             two_sum2(gs, gl, go);
         }
+        out_pair_done();
     }
     // target totals: P + u.G (flow) and the incoming sum (phase field); the
     // rest populations take the difference (conservation identities above),
@@ -554,54 +562,6 @@ __device__ __forceinline__ void collide_outputs(const DevParams& p, const CellSt
         phase_outputs_reduced<D>(p, s, gin, gsum_hi, gsum_lo, gout, dphiu_fn, gs, gl);
     else
         phase_rest(gsum_hi, gsum_lo, gs, gl, gout, C);
-}
-
-// The same outputs in two passes, phase field first: phase_outputs needs only
-// the closure (CellState without ew), so a kernel can run it before
-// flow_relax and reuse the staged pre-collision g for the moment
-// differences; flow_outputs then emits f'.  Each value is formed by the same
-// operations as in collide_outputs, and the rest populations accumulate the
-// moving ones in the same order, so the results are identical.
-template <int D, class GSrc, class Out>
-__device__ __forceinline__ void phase_outputs(const DevParams& p, const CellState& s, const GSrc& gin, float gsum_hi,
-                                              float gsum_lo, const Out& gout)
-{
-    constexpr int Q = Lat<D>::Q;
-    constexpr int C = Q / 2;
-    const float m15uu = -1.5f * s.uu;
-    float2 gs = f2(0.f, 0.f), gl = f2(0.f, 0.f);
-#pragma unroll
-    for (int a = 0; a < C; ++a) {
-        const int b = Q - 1 - a;
-        float2 gd, wgd;
-        pair_gamma<D>(s, a, m15uu, gd, wgd);
-        const float2 go = pair_phase<D>(p, s, a, wgd, f2(gin(a), gin(b)));
-        gout(a, go.x);
-        gout(b, go.y);
-        two_sum2(gs, gl, go);
-        out_pair_done();
-    }
-    phase_rest(gsum_hi, gsum_lo, gs, gl, gout, C);
-}
-template <int D, class Out, class DH>
-__device__ __forceinline__ void flow_outputs(const CellState& s, const DH& dh, const FlowMoments& m, const Out& fout)
-{
-    constexpr int Q = Lat<D>::Q;
-    constexpr int C = Q / 2;
-    const float m15uu = -1.5f * s.uu;
-    float2 fs = f2(0.f, 0.f);
-#pragma unroll
-    for (int a = 0; a < C; ++a) {
-        const int b = Q - 1 - a;
-        float2 gd, wgd;
-        pair_gamma<D>(s, a, m15uu, gd, wgd);
-        const float2 fo = pair_flow<D>(s, a, gd, wgd, f2(dh[a], dh[b]));
-        fout(a, fo.x);
-        fout(b, fo.y);
-        fs = add2(fs, fo);
-        out_pair_done();
-    }
-    flow_rest(s, m, fs, fout, C);
 }
 
 }  // namespace repro
