@@ -113,7 +113,7 @@ struct CodeLoad {
     template <int a>
     __device__ __forceinline__ void step() const
     {
-        if constexpr (a != C3) q[a] = __ldg(pulled<Walls, a>(base, C, P));
+        if constexpr (a != C3) q[a] = *pulled<Walls, a>(base, C, P);
     }
 };
 
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_fused3s_kernel(DevPa
 {
     extern __shared__ __align__(16) float smem16[];
     const ThreadGeo T = thread_geo();
-    for (int item = blockIdx.x; item < A.nitems; item += gridDim.x) {
+    for (int item = blockIdx.x + after_previous(); item < A.nitems; item += gridDim.x) {
         const int tile = item % (A.tiles_x * A.tiles_y);
         const int chunk = item / (A.tiles_x * A.tiles_y);
         const int z0 = chunk * A.chunk;
@@ -511,8 +511,7 @@ cudaError_t launch16(lbmp_handle* h, Cfg16& cfg)
     const LaunchShape L = launch_shape(h, A.tiles_x * A.tiles_y, h->grid.nz, cfg.per_sm, cfg.sms);
     A.chunk = L.chunk;
     A.nitems = L.nitems;
-    step_fused3s_kernel<St><<<L.grid, NT, kSmem16, h->stream>>>(h->dp, A, D);
-    return cudaGetLastError();
+    return launch_after(step_fused3s_kernel<St>, L, NT, kSmem16, h->stream, h->dp, A, D);
 }
 
 Cfg16 g_cfg_f16, g_cfg_bf16;

@@ -231,7 +231,7 @@ __device__ __forceinline__ void fused2_segment(const DevParams& p, const DirPtrs
         set_row2(R, p, y);
         float fr[Q2];
 #pragma unroll
-        for (int a = 0; a < Q2; ++a) fr[a] = __ldg(pulled2<SX>(D.fin, a, own, R));
+        for (int a = 0; a < Q2; ++a) fr[a] = *pulled2<SX>(D.fin, a, own, R);  // (plain: the set was written while this kernel was resident)
         stage_row<PR, SX>(p, D, own, side, tid, y + 1, gS + (cur ^ 1) * QG * TX2, sS, phiS + sN * RW, phiu,
                       uS + (cur ^ 1) * 2 * TX2);
         const off2 self = R.ys[1] + own.xs[1];
@@ -285,7 +285,7 @@ template <bool PR, bool SX>
 __global__ void __launch_bounds__(TX2, 7) step_fused2_kernel(DevParams p, Fused2Args A, DirPtrs2 D)
 {
     extern __shared__ float smem[];
-    for (int item = blockIdx.x; item < A.nitems; item += gridDim.x) {
+    for (int item = blockIdx.x + after_previous(); item < A.nitems; item += gridDim.x) {
         const int tile = item % A.tiles_x;
         const int y0 = (item / A.tiles_x) * A.chunk;
         fused2_segment<PR, SX ? kSymOn : kSymOff>(p, D, smem, tile * TX2, y0, min(y0 + A.chunk, p.ny), A.phiu);
@@ -396,13 +396,13 @@ cudaError_t launch_step_fused2(lbmp_handle* h)
     A.chunk = L.chunk;
     A.nitems = L.nitems;
     A.phiu = h->phiu;
+    const auto launch = [&](auto kernel) { return launch_after(kernel, L, TX2, kSmem2, h->stream, h->dp, A, D); };
     switch (k) {
-    case 0: step_fused2_kernel<false, false><<<L.grid, TX2, kSmem2, h->stream>>>(h->dp, A, D); break;
-    case 1: step_fused2_kernel<true, false><<<L.grid, TX2, kSmem2, h->stream>>>(h->dp, A, D); break;
-    case 2: step_fused2_kernel<false, true><<<L.grid, TX2, kSmem2, h->stream>>>(h->dp, A, D); break;
-    default: step_fused2_kernel<true, true><<<L.grid, TX2, kSmem2, h->stream>>>(h->dp, A, D); break;
+    case 0: return launch(step_fused2_kernel<false, false>);
+    case 1: return launch(step_fused2_kernel<true, false>);
+    case 2: return launch(step_fused2_kernel<false, true>);
+    default: return launch(step_fused2_kernel<true, true>);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t prepare_batch2(int device, bool reduced, bool sym)

@@ -158,8 +158,8 @@ __device__ __forceinline__ unsigned short pulled_code(const unsigned short* cons
 {
     const int cx = Lat<2>::cx(a), cy = Lat<2>::cy(a);
     bounced = (cy == 1 && C.lo) || (cy == -1 && C.hi);
-    if (bounced) return __ldg(at2s(q[Lat<2>::opp(a)], C.ys[1] + C.xs[1]));
-    return __ldg(at2s(q[a], C.ys[cy + 1] + C.xs[cx + 1]));
+    if (bounced) return *at2s(q[Lat<2>::opp(a)], C.ys[1] + C.xs[1]);
+    return *at2s(q[a], C.ys[cy + 1] + C.xs[cx + 1]);
 }
 
 // Decode the pulled g of one cell of row yy and sum its phi (hi, lo); Keep:
@@ -321,7 +321,7 @@ template <class St>
 __global__ void __launch_bounds__(TX2, 6) step_fused2s_kernel(DevParams p, Fused2sArgs A, DirPtrs2s D)
 {
     extern __shared__ __align__(16) float smem2s[];
-    for (int item = blockIdx.x; item < A.nitems; item += gridDim.x) {
+    for (int item = blockIdx.x + after_previous(); item < A.nitems; item += gridDim.x) {
         const int tile = item % A.tiles_x;
         const int y0 = (item / A.tiles_x) * A.chunk;
         fused2s_segment<St>(p, D, smem2s, tile * TX2, y0, min(y0 + A.chunk, p.ny));
@@ -431,8 +431,7 @@ struct Ops2s {
         D.rgin = h->g[s];
         D.rfout = h->f[d];
         D.rgout = h->g[d];
-        step_fused2s_kernel<St><<<L.grid, TX2, kSmem2s, h->stream>>>(h->dp, A, D);
-        return cudaGetLastError();
+        return launch_after(step_fused2s_kernel<St>, L, TX2, kSmem2s, h->stream, h->dp, A, D);
     }
     static cudaError_t prepare(int device)
     {

@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_fused3_kernel(DevPar
 {
     extern __shared__ float smem[];
     const ThreadGeo T = thread_geo();
-    for (int item = blockIdx.x; item < A.nitems; item += gridDim.x) {
+    for (int item = blockIdx.x + after_previous(); item < A.nitems; item += gridDim.x) {
         const int tile = item % (A.tiles_x * A.tiles_y);
         const int chunk = item / (A.tiles_x * A.tiles_y);
         const int z0 = p.zb + chunk * A.chunk;  // the updated planes [zb, ze) (all planes but a slab's ghosts)
@@ -539,8 +539,7 @@ cudaError_t LBMP_FUSED3_LAUNCH(lbmp_handle* h)
     const LaunchShape L = launch_shape(h, A.tiles_x * A.tiles_y, h->dp.ze - h->dp.zb, g_cfg.per_sm, g_cfg.sms);
     A.chunk = L.chunk;
     A.nitems = L.nitems;
-    step_fused3_kernel<<<L.grid, NT, kSmemBytes, h->stream>>>(h->dp, A, D);
-    return cudaGetLastError();
+    return launch_after(step_fused3_kernel, L, NT, kSmemBytes, h->stream, h->dp, A, D);
 }
 
 }  // namespace lbmp

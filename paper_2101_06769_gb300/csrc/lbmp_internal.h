@@ -109,6 +109,7 @@ inline int planes_per_item(const int* tiles, const int* nmarch, int n, long long
 // from the handle's options or the defaults.
 struct LaunchShape {
     int chunk, nitems, grid;
+    bool half_empty;  // the grid takes at most half of the GPU's slots
 };
 inline LaunchShape launch_shape(const lbmp_handle* h, int tiles, int nmarch, int per_sm, int sms)
 {
@@ -122,7 +123,32 @@ inline LaunchShape launch_shape(const lbmp_handle* h, int tiles, int nmarch, int
         L.chunk = planes_per_item(&tiles, &nmarch, 1, (long long)per_sm * sms);
     L.nitems = tiles * ((nmarch + L.chunk - 1) / L.chunk);
     L.grid = (int)(L.nitems < cap ? L.nitems : cap);
+    L.half_empty = 2LL * L.grid <= (long long)per_sm * sms;
     return L;
+}
+
+// Launch of a step kernel that begins with after_previous().  A grid that
+// leaves at least half of the GPU's slots empty is launched while the kernel
+// before it in the stream still runs (also as an edge of a captured graph): on
+// the legacy default stream a step of 64x256 D2Q9 cells takes 3.7 us instead
+// of 6.2, one of the 400x250 impact 8.4 instead of 10.2.  Fuller grids are not:
+// their early CTAs wait in the slots that the running step drains, which made
+// 1024x512 D2Q9 3 %, 64^3 D3Q27 3 % and 128x128x512 11 % slower.
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*kernel)(P...), const LaunchShape& L, unsigned block, size_t smem,
+                                cudaStream_t stream, const A&... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)L.grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = L.half_empty ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // bytes of one population set (f' or g) in the handle's storage form

@@ -165,7 +165,8 @@ __device__ __forceinline__ const E* pulled_g(const E* const* base, const Column&
     return at_cell(base[r], P.zs[cz + 1] + C.ys[cy + 1] + C.xs[cx + 1]);
 }
 
-// post-streaming values of the 27 directions of one cell into registers
+// post-streaming values of the 27 directions of one cell into registers (plain
+// loads: the set may have been written while this kernel was already resident)
 template <bool Walls>
 struct PullLoad {
     const float* const* base;
@@ -175,7 +176,7 @@ struct PullLoad {
     template <int a>
     __device__ __forceinline__ void step() const
     {
-        v[a] = __ldg(pulled<Walls, a>(base, C, P));
+        v[a] = *pulled<Walls, a>(base, C, P);
     }
 };
 
@@ -189,7 +190,7 @@ struct PullLoadG {
     template <int r>
     __device__ __forceinline__ void step() const
     {
-        v[r] = __ldg(pulled_g<Walls, r>(base, C, P));
+        v[r] = *pulled_g<Walls, r>(base, C, P);
     }
 };
 
