@@ -19,9 +19,10 @@
 //     the wall plane's phi instead of a second staging of that plane.
 // What bounds it: instruction issue (every value is decoded and encoded; DRAM
 // stands at a fifth of its rate) and the instruction cache.  It issues
-// 3045 instructions per cell (3553 when g codes were staged as 32-bit words and
-// the two population sets were emitted in two passes): 1.10 ms per step on the
-// 128x128x512 RT workload in FP16 (1.21 before), BF16 1.08 (1.18).  With the
+// 3002 instructions per cell (3553 when g codes were staged as 32-bit words, the
+// two population sets were emitted in two passes and divisions were the
+// compiler's): 1.09 ms per step on the 128x128x512 RT workload in FP16 (1.21
+// before), BF16 1.07 (1.18).  With the
 // ring's codes loaded beside the others (400 B of spills) 1.22, at four CTAs
 // per SM (500 B of spills) 1.12.
 #define LBMP_TILE_NS tile16

@@ -16,6 +16,14 @@
 // values (phi_sum_shifted) and keeps the decoded own values for the
 // collision.  Decoding, the collision and the encoding are those of the
 // reference pair (lbmp_kernels.cu), in the same order.
+// What bounds it: instruction issue (decoding and encoding; DRAM stands below
+// half of its rate).  So what does not change along the march is computed once
+// per segment (columns, staged slots, the row wrap without a division), code
+// and reference addresses of rows away from walls are emitted without the
+// bounce selection, and divisions and square roots of values known to be
+// normal take recip and root.  One step of 4096x2048: FP16 0.301 ms, BF16
+// 0.297 (0.343 and 0.341 with these left in the row loop); 1350x1021 BF16
+// 58.5 us (65.8).
 #include <type_traits>
 
 #include "lbmp_repro.cuh"
@@ -81,8 +89,8 @@ __device__ __forceinline__ void load_ref_row(const DevParams& p, const float* sr
     if (tid + TX2 < L) cp_async4(d + tid + TX2, base + xb);
 }
 
-// columns x-1, x, x+1 (periodic) and rows y+1, y, y-1 (periodic, or flagged
-// at a wall) of a cell, as offsets: index [c+1] is the upstream neighbour x - c
+// columns x+1, x, x-1 and rows y+1, y, y-1 (periodic) of a cell, as offsets:
+// index [c+1] is the upstream neighbour x - c.
 // 1: the offsets are unsigned byte offsets of the 2-byte codes (a pulled or
 // stored code's address is its array base plus one 32-bit sum); 0: signed
 // element indices scaled to 64 bits at every access
@@ -109,21 +117,28 @@ __device__ __forceinline__ E* at2s(E* base, off2s o)
 }
 __device__ __forceinline__ int elem2s(off2s o) { return (int)(o / kUnit2s); }
 
-struct Cell2 {
-    off2s xs[3], ys[3];
-    bool lo, hi;
+struct Col2s {
+    off2s xs[3];
 };
-
-__device__ __forceinline__ void set_cell2(Cell2& C, const DevParams& p, int x, int y)
+__device__ __forceinline__ void set_col2s(Col2s& C, int x, int nx)
 {
-    C.xs[0] = (off2s)(x + 1 == p.nx ? 0 : x + 1) * kUnit2s;
+    C.xs[0] = (off2s)(x + 1 == nx ? 0 : x + 1) * kUnit2s;
     C.xs[1] = (off2s)x * kUnit2s;
-    C.xs[2] = (off2s)(x == 0 ? p.nx - 1 : x - 1) * kUnit2s;
-    C.lo = !p.vert_periodic && y == 0;
-    C.hi = !p.vert_periodic && y == p.ny - 1;
-    C.ys[0] = (off2s)((y + 1 == p.ny ? 0 : y + 1) * p.nx) * kUnit2s;
-    C.ys[1] = (off2s)(y * p.nx) * kUnit2s;
-    C.ys[2] = (off2s)((y == 0 ? p.ny - 1 : y - 1) * p.nx) * kUnit2s;
+    C.xs[2] = (off2s)(x == 0 ? nx - 1 : x - 1) * kUnit2s;
+}
+struct Row2s {
+    off2s ys[3];
+    bool lo, hi;  // bottom / top row of a walled domain
+};
+// row y in [-1, ny] (its periodic image)
+__device__ __forceinline__ void set_row2s(Row2s& R, const DevParams& p, int y)
+{
+    y = y < 0 ? y + p.ny : (y >= p.ny ? y - p.ny : y);
+    R.lo = !p.vert_periodic && y == 0;
+    R.hi = !p.vert_periodic && y == p.ny - 1;
+    R.ys[0] = (off2s)((y + 1 == p.ny ? 0 : y + 1) * p.nx) * kUnit2s;
+    R.ys[1] = (off2s)(y * p.nx) * kUnit2s;
+    R.ys[2] = (off2s)((y == 0 ? p.ny - 1 : y - 1) * p.nx) * kUnit2s;
 }
 
 // the encoder of one cell's outputs at a cell offset: the codes at base +
@@ -150,57 +165,59 @@ struct EncCell2 {
     }
 };
 
-// code of the pulled population a of cell C, and whether it bounced at a wall
-// (then it is the opposite population of the cell itself); a is a
-// compile-time constant at every (unrolled) call site
-__device__ __forceinline__ unsigned short pulled_code(const unsigned short* const* q, int a, const Cell2& C,
-                                                      bool& bounced)
+// whether the pulled population a of a cell of row R bounced at a wall (then
+// it is the opposite population of the cell itself); Walls = false is the
+// path of every row that does not touch one
+template <bool Walls>
+__device__ __forceinline__ bool bounces(int a, const Row2s& R)
+{
+    return Walls && ((Lat<2>::cy(a) == 1 && R.lo) || (Lat<2>::cy(a) == -1 && R.hi));
+}
+// code values of the pulled pair (a, opp(a)) of the cell (C, R)
+template <bool Walls>
+__device__ __forceinline__ unsigned short pulled_code(const unsigned short* const* q, int a, const Col2s& C,
+                                                      const Row2s& R)
 {
     const int cx = Lat<2>::cx(a), cy = Lat<2>::cy(a);
-    bounced = (cy == 1 && C.lo) || (cy == -1 && C.hi);
-    if (bounced) return *at2s(q[Lat<2>::opp(a)], C.ys[1] + C.xs[1]);
-    return *at2s(q[a], C.ys[cy + 1] + C.xs[cx + 1]);
+    if (bounces<Walls>(a, R)) return *at2s(q[Lat<2>::opp(a)], R.ys[1] + C.xs[1]);
+    return *at2s(q[a], R.ys[cy + 1] + C.xs[cx + 1]);
+}
+// references of that pair's writers: entry e of the reference rows (row k in
+// slot k & 7, length L) around the logical row yy
+template <bool Walls>
+__device__ __forceinline__ float2 pair_refs(int a, const float* rows, int L, int yy, int e, const Row2s& R)
+{
+    const int cx = Lat<2>::cx(a), cy = Lat<2>::cy(a), b = Lat<2>::opp(a);
+    const auto row = [&](int k) { return rows + (k & (kRefRows - 1)) * L + e; };
+    return f2(bounces<Walls>(a, R) ? row(yy)[0] : row(yy - cy)[-cx], bounces<Walls>(b, R) ? row(yy)[0] : row(yy + cy)[cx]);
 }
 
 // Decode the pulled g of one cell of row yy and sum its phi (hi, lo); Keep:
 // also store the decoded values (= wr + wq, rounded once) at buf[a * TX2].
-// yy is a logical row (y0 - 1 .. y1; not a ghost row beyond a wall): the
-// codes are read from its periodic image, the references from the slots of
-// the logical rows yy-1, yy, yy+1 in RG; e is the cell's entry in a
-// reference row.
-template <class St, bool Keep>
-__device__ __forceinline__ float2 decode_g_cell(const DevParams& p, const DirPtrs2s& D, const float* RG, int yy,
-                                                int x, int e, float* buf)
+// yy is a logical row (y0 - 1 .. y1; not a ghost row beyond a wall) with
+// row R; e is the cell's entry in a reference row.
+template <bool Walls, class St, bool Keep>
+__device__ __forceinline__ float2 decode_g_cell(const DirPtrs2s& D, const float* RG, int yy, const Col2s& C,
+                                                const Row2s& R, int e, float* buf)
 {
-    Cell2 C;
-    set_cell2(C, p, x, pmod(yy, p.ny));
-    const float* R0 = RG + (yy & (kRefRows - 1)) * GW + e;
-    const auto code_and_ref = [&](int a, float& c, float& r) {
-        bool bounced;
-        const int cx = Lat<2>::cx(a), cy = Lat<2>::cy(a);
-        c = St::dec(pulled_code(D.gin, a, C, bounced));
-        r = bounced ? R0[0] : RG[((yy - cy) & (kRefRows - 1)) * GW + e - cx];
-    };
-    float hi, lo;
+    const float rest = wint<2>(C2) * RG[(yy & (kRefRows - 1)) * GW + e];
+    if (Keep) buf[C2 * TX2] = rest;
+    float2 phi;
     phi_sum_shifted<2>(
-        [&]() {
-            const float v = wint<2>(C2) * R0[0];
-            if (Keep) buf[C2 * TX2] = v;
-            return v;
-        },
+        [&]() { return rest; },
         [&](int a, float2& wr, float2& wq) {
-            float2 q, R;
-            code_and_ref(a, q.x, R.x);
-            code_and_ref(Q2 - 1 - a, q.y, R.y);
-            decode_pair<2, St>(a, R, q, wr, wq);
+            const int b = Lat<2>::opp(a);
+            const float2 q = f2(St::dec(pulled_code<Walls>(D.gin, a, C, R)), St::dec(pulled_code<Walls>(D.gin, b, C, R)));
+            const float2 r = pair_refs<Walls>(a, RG, GW, yy, e, R);
+            decode_pair<2, St>(a, r, q, wr, wq);
             if (Keep) {
-                const float2 v = decode_pair<2, St>(a, R, q);
+                const float2 v = decode_pair<2, St>(a, r, q);
                 buf[a * TX2] = v.x;
-                buf[(Q2 - 1 - a) * TX2] = v.y;
+                buf[b * TX2] = v.y;
             }
         },
-        hi, lo);
-    return make_float2(hi, lo);
+        phi.x, phi.y);
+    return phi;
 }
 
 // rows [y0, y1) of the segment starting at x0.  One barrier per row: the
@@ -219,8 +236,9 @@ __device__ __forceinline__ void fused2s_segment(const DevParams& p, const DirPtr
     float* RG = RF + kRefRows * RW;            // [8][GW] g references
     float2* phiS = (float2*)(RG + kRefRows * GW);  // [4][RW]
     const int tid = threadIdx.x;
-    const int x_own = pmod(x0 + tid, p.nx);
-    const int x_side = pmod(tid == 0 ? x0 - 1 : x0 + TX2, p.nx);
+    Col2s own, side;
+    set_col2s(own, pmod(x0 + tid, p.nx), p.nx);
+    set_col2s(side, pmod(tid == 0 ? x0 - 1 : x0 + TX2, p.nx), p.nx);
     const int e_side = tid == 0 ? 1 : TX2 + 2;  // side cell's entry in a g reference row
     const bool valid = x0 + tid < p.nx;
     const int fa = pmod(x0 - 1 + tid, p.nx), fb = pmod(x0 - 1 + tid + TX2, p.nx);
@@ -236,8 +254,18 @@ __device__ __forceinline__ void fused2s_segment(const DevParams& p, const DirPtr
             prow[tid + 1] = wrow[tid + 1];
             return;
         }
-        if (tid < 2) prow[tid == 0 ? 0 : RW - 1] = decode_g_cell<St, false>(p, D, RG, yy, x_side, e_side, nullptr);
-        prow[tid + 1] = decode_g_cell<St, true>(p, D, RG, yy, x_own, tid + 2, gbuf + tid);
+        Row2s R;
+        set_row2s(R, p, yy);
+        const auto decode = [&](auto walls) {
+            constexpr bool W = decltype(walls)::value;
+            if (tid < 2)
+                prow[tid == 0 ? 0 : RW - 1] = decode_g_cell<W, St, false>(D, RG, yy, side, R, e_side, nullptr);
+            prow[tid + 1] = decode_g_cell<W, St, true>(D, RG, yy, own, R, tid + 2, gbuf + tid);
+        };
+        if (R.lo || R.hi)  // uniform across the CTA
+            decode(std::true_type{});
+        else
+            decode(std::false_type{});
     };
     // references for the first rows: g rows y0-2 .. y0+2, f' rows y0-1 .. y0+1
     for (int k = y0 - 2; k <= y0 + 2; ++k) load_ref_row(p, D.rgin, k, RG, GW, ga, gb, tid);
@@ -259,55 +287,59 @@ __device__ __forceinline__ void fused2s_segment(const DevParams& p, const DirPtr
         load_ref_row(p, D.rgin, y + 3, RG, GW, ga, gb, tid);
         load_ref_row(p, D.rfin, y + 2, RF, RW, fa, fb, tid);
         cp_async_commit();
-        Cell2 C;
-        set_cell2(C, p, x_own, y);
-        unsigned short q[Q2];
-        bool bq[Q2];
-#pragma unroll
-        for (int a = 0; a < Q2; ++a)
-            if (a != C2) q[a] = pulled_code(D.fin, a, C, bq[a]);
-        stage_g(y + 1, gS + (cur ^ 1) * Q2 * TX2, sN, sC);
+        Row2s R;
+        set_row2s(R, p, y);
         repro::FlowMoments m;
-        {
-            const float* R0 = RF + (y & (kRefRows - 1)) * RW + tid + 1;
-            float fr[Q2];
+        const bool wall = R.lo || R.hi;  // uniform across the CTA
+        unsigned short q[Q2];
+        const auto load_f = [&](auto walls) {
 #pragma unroll
-            for (int a = 0; a < Q2; ++a) {
-                const int cx = Lat<2>::cx(a), cy = Lat<2>::cy(a);
-                if (a == C2) {
-                    fr[a] = wint<2>(C2) * R0[0];
-                } else {
-                    const float R = bq[a] ? R0[0] : RF[((y - cy) & (kRefRows - 1)) * RW + tid + 1 - cx];
-                    fr[a] = dec_value<2, St>(a, St::dec(q[a]), R);
-                }
+            for (int a = 0; a < Q2; ++a)
+                if (a != C2) q[a] = pulled_code<decltype(walls)::value>(D.fin, a, own, R);
+        };
+        const auto decode_f = [&](auto walls) {
+            float fr[Q2];
+            fr[C2] = wint<2>(C2) * RF[(y & (kRefRows - 1)) * RW + tid + 1];
+#pragma unroll
+            for (int a = 0; a < C2; ++a) {
+                const int b = Lat<2>::opp(a);
+                const float2 v = decode_pair<2, St>(
+                    a, pair_refs<decltype(walls)::value>(a, RF, RW, y, tid + 1, R), f2(St::dec(q[a]), St::dec(q[b])));
+                fr[a] = v.x;
+                fr[b] = v.y;
             }
             repro::flow_moments<2>(m, fr);
-        }
+        };
+        // f' codes first, decoded after the g of row y+1
+        if (wall)
+            load_f(std::true_type{});
+        else
+            load_f(std::false_type{});
+        stage_g(y + 1, gS + (cur ^ 1) * Q2 * TX2, sN, sC);
+        if (wall)
+            decode_f(std::true_type{});
+        else
+            decode_f(std::false_type{});
         cp_async_wait_all();
         __syncthreads();
         if (valid) {
-            float nh[Q2], nl[Q2];
-#pragma unroll
-            for (int a = 0; a < Q2; ++a) {
+            const auto nb = [&](int a) {  // phi of the stencil's neighbour a
                 const int cy = Lat<2>::cy(a);
-                const float2 v = phiS[(cy < 0 ? sP : (cy == 0 ? sC : sN)) * RW + tid + 1 + Lat<2>::cx(a)];
-                nh[a] = v.x;
-                nl[a] = v.y;
-            }
-            float grad[3], lap;
-            repro::stencil_from_nb<2>(nh, nl, grad, lap);
+                return phiS[(cy < 0 ? sP : (cy == 0 ? sC : sN)) * RW + tid + 1 + Lat<2>::cx(a)];
+            };
+            const float2 c = nb(C2);
+            float grad[3], lap, inv_rho, nu, dh[27];
+            repro::stencil_from<2>(nb, c, grad, lap);
             repro::CellState s;
-            float dh[27];
-            float inv_rho, nu;
-            repro::flow_closure<2>(p, nh[C2], grad, lap, m, s, inv_rho, nu);
+            repro::flow_closure<2>(p, c.x, grad, lap, m, s, inv_rho, nu);
             repro::flow_relax<2>(m, s, inv_rho, nu, dh);
-            const off2s self = C.ys[1] + C.xs[1];
+            const off2s self = R.ys[1] + own.xs[1];
             const GFromStrided gi{gS + cur * Q2 * TX2 + tid, TX2};
             float off_f, off_g;
             repro::rest_offsets<2, St>(p, s, dh, gi, off_f, off_g);
             const EncCell2<St> fo{D.fout, D.rfout, self, off_f, 0.f, code_seed(p, elem2s(self), 0)};
             const EncCell2<St> go{D.gout, D.rgout, self, off_g, 0.f, code_seed(p, elem2s(self), 1)};
-            repro::collide_outputs<2>(p, s, repro::DhArray{dh}, m, gi, nh[C2], nl[C2], fo, go);
+            repro::collide_outputs<2>(p, s, repro::DhArray{dh}, m, gi, c.x, c.y, fo, go);
         }
     }
     __syncthreads();

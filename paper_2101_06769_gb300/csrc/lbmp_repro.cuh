@@ -155,14 +155,14 @@ __device__ __forceinline__ float flow_closure(const DevParams& p, float phi, con
                                               const FlowMoments& m, CellState& s, float& inv_rho, float& nu)
 {
     const float rho = p.rho_l + p.drho * phi;
-    inv_rho = 1.0f / rho;
+    inv_rho = recip(rho);
     if (p.flags & kFlagDynamicVisc)
         nu = (p.eta_l + (p.eta_h - p.eta_l) * phi) * inv_rho;
     else
         nu = p.nu_h + (p.nu_l - p.nu_h) * (1.0f - phi);
     // interface normal, chemical potential, force
     const float g2 = grad[0] * grad[0] + grad[1] * grad[1] + (D == 3 ? grad[2] * grad[2] : 0.f);
-    const float inv_g = 1.0f / fmaxf(sqrtf(g2), 1e-4f);
+    const float inv_g = recip(fmaxf(root(fmaxf(g2, 1e-12f)), 1e-4f));
     const float mu = p.beta2 * phi * (phi - 1.0f) * (2.0f * phi - 1.0f) - p.kappa * lap;
     float F[3];
     F[0] = mu * grad[0];
@@ -198,7 +198,7 @@ __device__ __forceinline__ float flow_closure(const DevParams& p, float phi, con
 template <int D>
 __device__ __forceinline__ void flow_relax(const FlowMoments& m, CellState& s, float inv_rho, float nu, float dh[27])
 {
-    const float omega = 1.0f / (3.0f * nu + 0.5f);
+    const float omega = recip(3.0f * nu + 0.5f);
     const float om1 = 1.0f - omega;
     const float ux = s.u[0], uy = s.u[1], uz = s.u[2];
     float V[3];
@@ -369,16 +369,10 @@ __device__ __forceinline__ void rest_offsets(const DevParams& p, const CellState
 // (c -> -c, same weight): (a, opp(a)) are the two lanes of the paired FP32
 // arithmetic, and the shared factors (c.u, (c.u)^2, c.G, c.F, c.n) are
 // computed once per pair.
-// dh source: the register array of flow_collide, or a copy parked in shared
-// memory (strided per thread) to lower register pressure in the output loop
+// dh source: the register array of flow_collide
 struct DhArray {
     const float* v;
     __device__ __forceinline__ float operator[](int a) const { return v[a]; }
-};
-struct DhStrided {
-    const float* base;
-    int stride;
-    __device__ __forceinline__ float operator[](int a) const { return base[a * stride]; }
 };
 
 // Per-pair pieces of the outputs.  Direction a < Q/2 and its opposite
