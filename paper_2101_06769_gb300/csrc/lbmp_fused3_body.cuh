@@ -172,6 +172,16 @@ __device__ __forceinline__ void stage_finish(int tid, int oslot, int rslot, cons
 // written and read by the same thread, and the phi of plane z+1 goes to the
 // slot that was last read before the previous plane's barrier.  Ends with a
 // barrier, so the caller may reuse shared memory afterwards.
+//
+// Ahead: f'(z+1) is loaded to registers once the moments of f'(z) are formed, so
+// its latency runs beside the collision and the stores of plane z.  The 27
+// values live across the collision: 168 registers, three CTAs per SM.  Against
+// four CTAs without, on D3Q27 FP32: 128x128x512 0.736 -> 0.715 ms, 384x384x192
+// 2.58 -> 2.52 ms, 160^3 0.377 -> 0.363 ms; where a step is a few planes per
+// CTA the fourth CTA is worth more (48^3 14.7 -> 16.5 us, 32^3 6.9 -> 7.4 us),
+// and so it is to batches (3.7 M cells 324 -> 330 us) and the reduced phase
+// lattice (0.447 -> 0.458 ms).  At two CTAs per SM 0.760 ms.
+template <bool Ahead>
 __device__ __forceinline__ void fused_segment(const DevParams& p, const DirPtrs& Dp, const ThreadGeo& T, float* smem,
                                               int x0, int y0, int z0, int z1, float* __restrict__ phiu)
 {
@@ -192,6 +202,18 @@ __device__ __forceinline__ void fused_segment(const DevParams& p, const DirPtrs&
     stage_finish(tid, oslot, rslot, gS + QG * NT, rS, phiS);
     stage_issue(p, Dp, own, ring, tid, rslot, z0, gS, rS, phiu, uS, phiS + PLANE);
     stage_finish(tid, oslot, rslot, gS, rS, phiS + PLANE);
+    float fr[Q3];
+    const auto pull_f = [&](const Plane& P) {
+        if (P.lo || P.hi)
+            Unroll<Q3>::run(PullLoad<true>{Dp.fin, own, P, fr});
+        else
+            Unroll<Q3>::run(PullLoad<false>{Dp.fin, own, P, fr});
+    };
+    if constexpr (Ahead) {
+        Plane P;
+        set_plane(P, p, z0);
+        pull_f(P);
+    }
     LayerSums below, here;
     __syncthreads();
     layer(0, below);
@@ -199,18 +221,21 @@ __device__ __forceinline__ void fused_segment(const DevParams& p, const DirPtrs&
     __syncthreads();
     for (int z = z0; z < z1; ++z) {
         const int cur = (z - z0) & 1;
-        // g(z+1) and the ring copies in flight while f'(z) is loaded
+        // g(z+1) and the ring copies in flight while f'(z) is loaded, or (Ahead)
+        // while the moments of the f'(z) loaded one plane ago are formed
         stage_issue(p, Dp, own, ring, tid, rslot, z + 1, gS + (cur ^ 1) * QG * NT, rS, phiu, uS + (cur ^ 1) * 3 * NT,
                     phiS + cur * PLANE);
         Plane P;
         set_plane(P, p, z);
         FlowMoments m;
-        {
-            float fr[Q3];
-            if (P.lo || P.hi)
-                Unroll<Q3>::run(PullLoad<true>{Dp.fin, own, P, fr});
-            else
-                Unroll<Q3>::run(PullLoad<false>{Dp.fin, own, P, fr});
+        if constexpr (Ahead) {
+            flow_moments<3>(m, fr);
+            stage_finish(tid, oslot, rslot, gS + (cur ^ 1) * QG * NT, rS, phiS + cur * PLANE);
+            Plane N;
+            set_plane(N, p, z + 1 < z1 ? z + 1 : z);
+            pull_f(N);
+        } else {
+            pull_f(P);
             stage_finish(tid, oslot, rslot, gS + (cur ^ 1) * QG * NT, rS, phiS + cur * PLANE);
             flow_moments<3>(m, fr);
         }
@@ -236,7 +261,9 @@ __device__ __forceinline__ void fused_segment(const DevParams& p, const DirPtrs&
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_fused3_kernel(DevParams p, FusedArgs A, DirPtrs Dp)
+template <bool Ahead>
+__global__ void __launch_bounds__(NT, Ahead ? 3 : LBMP_FUSED_MINB)
+    step_fused3_kernel(DevParams p, FusedArgs A, DirPtrs Dp)
 {
     extern __shared__ float smem[];
     const ThreadGeo T = thread_geo();
@@ -244,7 +271,7 @@ __global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_fused3_kernel(DevPar
         const int tile = item % (A.tiles_x * A.tiles_y);
         const int chunk = item / (A.tiles_x * A.tiles_y);
         const int z0 = p.zb + chunk * A.chunk;  // the updated planes [zb, ze) (all planes but a slab's ghosts)
-        fused_segment(p, Dp, T, smem, (tile % A.tiles_x) * TX, (tile / A.tiles_x) * TY, z0,
+        fused_segment<Ahead>(p, Dp, T, smem, (tile % A.tiles_x) * TX, (tile / A.tiles_x) * TY, z0,
                       min(z0 + A.chunk, p.ze), A.phiu);
     }
 }
@@ -281,7 +308,7 @@ __global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_batchg3_kernel(const
     for (int item = blockIdx.x; item < M.items; item += gridDim.x) {
         const int tile = item % tiles;
         const int z0 = M.p.zb + (item / tiles) * M.chunk;
-        fused_segment(M.p, M.D, T, smem, (tile % M.tiles_x) * TX, (tile / M.tiles_x) * TY, z0,
+        fused_segment<false>(M.p, M.D, T, smem, (tile % M.tiles_x) * TX, (tile / M.tiles_x) * TY, z0,
                       min(z0 + M.chunk, M.p.ze), M.phiu);
     }
 }
@@ -381,7 +408,25 @@ struct LaunchCfg {
     int device = -1;
     int per_sm = 0, sms = 0;
 };
-LaunchCfg g_cfg;
+LaunchCfg g_cfg[2];  // without and with f' loaded ahead
+
+cudaError_t step_config(const lbmp_handle* h, bool ahead)
+{
+    LaunchCfg& cfg = g_cfg[ahead];
+    if (cfg.device == h->device) return cudaSuccess;
+    const auto kernel = ahead ? step_fused3_kernel<LBMP_FUSED_AHEAD != 0> : step_fused3_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0, sms = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, kSmemBytes);
+    if (e != cudaSuccess) return e;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (e != cudaSuccess) return e;
+    cfg.per_sm = per_sm > 0 ? per_sm : 1;
+    cfg.sms = sms;
+    cfg.device = h->device;
+    return cudaSuccess;
+}
 
 }  // namespace
 
@@ -518,28 +563,28 @@ const Batch3Ops LBMP_BATCH3_OPS = {TX, TY, prepare_batch, nullptr, launch_batch_
 
 cudaError_t LBMP_FUSED3_LAUNCH(lbmp_handle* h)
 {
-    if (g_cfg.device != h->device) {
-        cudaError_t e = cudaFuncSetAttribute(step_fused3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kSmemBytes);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_fused3_kernel, NT, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-        if (e != cudaSuccess) return e;
-        g_cfg.per_sm = per_sm > 0 ? per_sm : 1;
-        g_cfg.sms = sms;
-        g_cfg.device = h->device;
-    }
+    cudaError_t e = step_config(h, false);
+    if (e != cudaSuccess) return e;
     const DirPtrs D = dir_ptrs(h);
     FusedArgs A;
     A.phiu = h->phiu;
     A.tiles_x = (h->grid.nx + TX - 1) / TX;
     A.tiles_y = (h->grid.ny + TY - 1) / TY;
-    const LaunchShape L = launch_shape(h, A.tiles_x * A.tiles_y, h->dp.ze - h->dp.zb, g_cfg.per_sm, g_cfg.sms);
+    const int tiles = A.tiles_x * A.tiles_y, nmarch = h->dp.ze - h->dp.zb;
+#if LBMP_FUSED_AHEAD
+    e = step_config(h, true);
+    if (e != cudaSuccess) return e;
+    const int per_sm[2] = {g_cfg[0].per_sm, g_cfg[1].per_sm};
+    bool ahead;
+    const LaunchShape L = launch_shape_ahead(h, tiles, nmarch, per_sm, g_cfg[0].sms, ahead);
+    const auto kernel = ahead ? step_fused3_kernel<true> : step_fused3_kernel<false>;
+#else
+    const LaunchShape L = launch_shape(h, tiles, nmarch, g_cfg[0].per_sm, g_cfg[0].sms);
+    const auto kernel = step_fused3_kernel<false>;
+#endif
     A.chunk = L.chunk;
     A.nitems = L.nitems;
-    return launch_after(step_fused3_kernel, L, NT, kSmemBytes, h->stream, h->dp, A, D);
+    return launch_after(kernel, L, NT, kSmemBytes, h->stream, h->dp, A, D);
 }
 
 }  // namespace lbmp

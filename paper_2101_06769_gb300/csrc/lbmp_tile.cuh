@@ -34,6 +34,11 @@ namespace LBMP_TILE_NS {
 #ifndef LBMP_FUSED_RINGREG
 #define LBMP_FUSED_RINGREG 0
 #endif
+// 1: the unit also builds the step that loads f'(z+1) to registers before the
+// collision of plane z
+#ifndef LBMP_FUSED_AHEAD
+#define LBMP_FUSED_AHEAD 0
+#endif
 // E > 0: the column and plane offsets are unsigned byte offsets of E-byte
 // populations, so a pulled value's address is its array base plus one
 // 32-bit sum (every array below 4 GiB); 0: signed element indices, scaled
