@@ -37,6 +37,8 @@ struct AAPtrs {
     float* g[Q3];  // and of the single g set
 };
 
+constexpr MarchCost kCost = {8.0, 0.4, 0.0};
+
 struct AAArgs {
     int tiles_x, tiles_y, chunk, nitems;
     const float* phi;  // phi hi [0, N), lo [N, 2N) from the phi pass
@@ -254,7 +256,7 @@ cudaError_t launch_aa(lbmp_handle* h)
     A.tiles_x = (h->grid.nx + TX - 1) / TX;
     A.tiles_y = (h->grid.ny + TY - 1) / TY;
     A.phi = h->phi;
-    const LaunchShape L = launch_shape(h, A.tiles_x * A.tiles_y, h->grid.nz, g_aa.per_sm[Odd ? 1 : 0], g_aa.sms);
+    const LaunchShape L = launch_shape(h, kCost, A.tiles_x * A.tiles_y, h->grid.nz, g_aa.per_sm[Odd ? 1 : 0], g_aa.sms);
     A.chunk = L.chunk;
     A.nitems = L.nitems;
     step_aa_kernel<Odd><<<L.grid, NT, kSmemAA, h->stream>>>(h->dp, A, D);

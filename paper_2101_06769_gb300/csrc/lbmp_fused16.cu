@@ -81,6 +81,8 @@ struct DirPtrs16 {
     float* rgout;
 };
 
+constexpr MarchCost kCost = {6.0, 1.25, 0.0};
+
 struct FusedArgs16 {
     int tiles_x, tiles_y, chunk, nitems;
 };
@@ -509,7 +511,7 @@ cudaError_t launch16(lbmp_handle* h, Cfg16& cfg)
     FusedArgs16 A;
     A.tiles_x = (h->grid.nx + TX - 1) / TX;
     A.tiles_y = (h->grid.ny + TY - 1) / TY;
-    const LaunchShape L = launch_shape(h, A.tiles_x * A.tiles_y, h->grid.nz, cfg.per_sm, cfg.sms);
+    const LaunchShape L = launch_shape(h, kCost, A.tiles_x * A.tiles_y, h->grid.nz, cfg.per_sm, cfg.sms);
     A.chunk = L.chunk;
     A.nitems = L.nitems;
     return launch_after(step_fused3s_kernel<St>, L, NT, kSmem16, h->stream, h->dp, A, D);

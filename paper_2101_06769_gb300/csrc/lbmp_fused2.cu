@@ -353,6 +353,8 @@ __global__ void __launch_bounds__(TX2) step_batch2_kernel(const BatchDomain* __r
 int g_f2_dev[4] = {-1, -1, -1, -1}, g_f2_per_sm[4] = {0, 0, 0, 0}, g_f2_sms[4] = {0, 0, 0, 0},
     g_b2_dev[4] = {-1, -1, -1, -1}, g_b2_cap[4] = {0, 0, 0, 0};
 
+constexpr MarchCost kCost = {3.0, 1.25, 6.0};
+
 cudaError_t setup_kernel(const void* fn, int device, int& dev_cached, int& per_sm_out, int& sms_out)
 {
     if (dev_cached == device) return cudaSuccess;
@@ -392,7 +394,7 @@ cudaError_t launch_step_fused2(lbmp_handle* h)
     }
     Fused2Args A;
     A.tiles_x = (h->grid.nx + TX2 - 1) / TX2;
-    const LaunchShape L = launch_shape(h, A.tiles_x, h->grid.ny, g_f2_per_sm[k], g_f2_sms[k]);
+    const LaunchShape L = launch_shape(h, kCost, A.tiles_x, h->grid.ny, g_f2_per_sm[k], g_f2_sms[k]);
     A.chunk = L.chunk;
     A.nitems = L.nitems;
     A.phiu = h->phiu;

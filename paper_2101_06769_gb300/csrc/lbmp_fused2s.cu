@@ -345,6 +345,8 @@ __device__ __forceinline__ void fused2s_segment(const DevParams& p, const DirPtr
     __syncthreads();
 }
 
+constexpr MarchCost kCost = {3.0, 0.4, 15.0};
+
 struct Fused2sArgs {
     int tiles_x, chunk, nitems;
 };
@@ -454,7 +456,7 @@ struct Ops2s {
         const int s = h->parity, d = 1 - h->parity;
         Fused2sArgs A;
         A.tiles_x = (h->grid.nx + TX2 - 1) / TX2;
-        const LaunchShape L = launch_shape(h, A.tiles_x, h->grid.ny, step_cfg.per_sm, step_cfg.sms);
+        const LaunchShape L = launch_shape(h, kCost, A.tiles_x, h->grid.ny, step_cfg.per_sm, step_cfg.sms);
         A.chunk = L.chunk;
         A.nitems = L.nitems;
         DirPtrs2s D;

@@ -408,6 +408,8 @@ struct LaunchCfg {
     int device = -1;
     int per_sm = 0, sms = 0;
 };
+constexpr MarchCost kCost = PR ? MarchCost{8.0, 1.0, 6.0} : kCostFp32[0];
+
 LaunchCfg g_cfg[2];  // without and with f' loaded ahead
 
 cudaError_t step_config(const lbmp_handle* h, bool ahead)
@@ -579,7 +581,7 @@ cudaError_t LBMP_FUSED3_LAUNCH(lbmp_handle* h)
     const LaunchShape L = launch_shape_ahead(h, tiles, nmarch, per_sm, g_cfg[0].sms, ahead);
     const auto kernel = ahead ? step_fused3_kernel<true> : step_fused3_kernel<false>;
 #else
-    const LaunchShape L = launch_shape(h, tiles, nmarch, g_cfg[0].per_sm, g_cfg[0].sms);
+    const LaunchShape L = launch_shape(h, kCost, tiles, nmarch, g_cfg[0].per_sm, g_cfg[0].sms);
     const auto kernel = step_fused3_kernel<false>;
 #endif
     A.chunk = L.chunk;

@@ -312,7 +312,7 @@ cudaError_t launch_step_fused_bulk(lbmp_handle* h)
     BulkArgs A;
     A.tiles_x = (h->grid.nx + TX - 1) / TX;
     A.tiles_y = (h->grid.ny + TY - 1) / TY;
-    const LaunchShape L = launch_shape(h, A.tiles_x * A.tiles_y, h->grid.nz, g_bulk.per_sm, g_bulk.sms);
+    const LaunchShape L = launch_shape(h, kCostFp32[0], A.tiles_x * A.tiles_y, h->grid.nz, g_bulk.per_sm, g_bulk.sms);
     A.chunk = L.chunk;
     A.nitems = L.nitems;
     step_fused3b_kernel<<<L.grid, NT, smem, h->stream>>>(h->dp, A, D);

@@ -45,9 +45,8 @@ struct lbmp_handle {
     int opt_ctas;      // LBMP_OPT_CTAS_PER_SM: resident CTAs per SM of the grid, 0 = occupancy maximum
     int opt_tile;      // LBMP_OPT_TILE: tile shape of the FP32 D3Q27 fused kernel (0 32x4, 1 16x8, 2 8x16)
     int probe[3];
-    // FP32 D3Q27 step: kernel and launch shape last worked out, for the planes
-    // and options in shape_for
-    int shape[3], shape_for[3];
+    // planes per work item and kernel last chosen for the step, and what for
+    int shape[2], shape_for[6];
     // step graphs (lbmp_step): kStepGraph steps captured from each starting
     // parity, for the launch options in graph_key; warm once a plain step
     // ran with those options (the kernels' one-time set-up is not captured)
@@ -72,21 +71,120 @@ struct BatchDomain {
     int tiles_x, tiles_y, chunk, item_begin, items;
 };
 
-// Default planes (rows in 2-D) per work item (the FP32 D3Q27 step of one domain
-// has a rule of its own, launch_shape_ahead) of `n` domains stepped by one
-// launch, domain k with tiles[k] tiles marching through nmarch[k] planes, on
-// `slots` resident CTAs.  Where 8 or more planes per item leave 2.5 rounds
-// of the full grid, the largest power-of-two part of the longest domain that
-// does: each item stages two planes more than it updates, so longer items win
-// until the rounds get coarse (128x128x512 RT: 32 planes 0.730 ms per step,
-// 16 planes 0.731, 64 planes 0.757).  Smaller work cannot fill 2.5 rounds;
-// there the time is about rounds x (planes + 1.5) x (0.7 + occupancy), the
-// stages of one item times a stage's latency, which grows with the number of
-// CTAs that share an SM, and the rule takes the planes that make it smallest.
-// Measured in us per step, 8 planes -> the rule's choice: D2Q9 64x256
-// 8.6 -> 3.5 (1 row), 400x250 10.0 -> 6.4 (2), 1024x512 17.1 -> 15.2 (4),
-// 2048x1024 65.4 -> 61.2 (16); D3Q27 32^3 18.7 -> 7.3 (1 plane), 48^3
-// 18.6 -> 14.5 (2), 64^3 31.4 -> 26.3 (4).
+// Estimated time of a launch of `tiles` tiles marching through `nmarch` planes
+// (rows in 2-D) in items of `chunk` planes, on per_sm CTAs of each of `sms` SMs,
+// in units of its own kernel: a plane takes `plane` + the CTAs that share the
+// SM, an item `extra` planes more than it updates, a grid that is not launched
+// early (launch_after) `gap`.  In the first rounds the slots run in step, so the
+// time is that of the rounds, the last one with the CTAs that are left; later
+// the slots have drifted apart and the time tends to the mean load.
+struct MarchCost {
+    double plane, extra, gap;
+};
+inline double march_time(const MarchCost& m, int tiles, int nmarch, int chunk, int per_sm, int sms)
+{
+    const int per_tile = (nmarch + chunk - 1) / chunk;
+    const long long slots = (long long)per_sm * sms, items = (long long)tiles * per_tile;
+    const long long rounds = (items + slots - 1) / slots;
+    const double full = m.plane + per_sm, last = m.plane + (double)(items - (rounds - 1) * slots) / sms;
+    const double in_step = (chunk + m.extra) * ((double)(rounds - 1) * full + last);
+    const double mean = (double)tiles * (nmarch + m.extra * per_tile) / (double)slots * full;
+    const double least = (chunk + m.extra) * (rounds == 1 ? last : full);
+    const double w = std::exp(-0.4 * (double)(rounds - 1));
+    return w * in_step + (1.0 - w) * (mean > least ? mean : least) + (2 * items > slots ? m.gap : 0.0);
+}
+constexpr int kLongestItem = 64;  // planes (items of up to 72 were measured)
+
+// Launch shape of a persistent fused kernel over `tiles` tiles marching
+// through `nmarch` planes (rows in 2-D): planes per work item and grid size,
+// from the handle's options or the shape with the least estimated time.
+struct LaunchShape {
+    int chunk, nitems, grid;
+    bool half_empty;  // the grid takes at most half of the GPU's slots
+};
+inline LaunchShape shape_of(const lbmp_handle* h, int tiles, int nmarch, int chunk, int per_sm, int sms)
+{
+    const long long cap = (long long)((h->opt_ctas > 0 && h->opt_ctas < per_sm) ? h->opt_ctas : per_sm) * sms;
+    LaunchShape L;
+    L.chunk = chunk < nmarch ? chunk : nmarch;
+    L.nitems = tiles * ((nmarch + L.chunk - 1) / L.chunk);
+    L.grid = (int)(L.nitems < cap ? L.nitems : cap);
+    L.half_empty = 2LL * L.grid <= (long long)per_sm * sms;
+    return L;
+}
+
+// n kernels that compute the same step: cost[k] in units that compare, per_sm[k]
+// the CTAs each reaches.  The choice is kept in the handle until the options it
+// was made for change (64 estimates, 2 us of host time).  The constants of each
+// kernel are the best of a grid over 64 (FP32 D3Q27: 238) domains of 2e4 to 1e7
+// (2e7) cells, each measured with every chunk of a dense set.  On 50 other
+// domains of that range, time against the rule before (the longest axis halved
+// until 2.5 rounds of the grid are full, else the best of a simpler estimate),
+// on average and at worst: D3Q27 FP16 0.949 and 1.04, BF16 0.947 and 1.01, FP32
+// in place 0.984 and 1.01, reduced phase lattice 0.989 and 1.01, D2Q9 FP32 0.978
+// and 1.05, reduced 0.988 and 1.08, FP16 and BF16 0.930 and 1.01.  The best
+// measured chunks of the first set: 0.955, 0.981, 0.987, 0.972 and 0.946 for
+// 16-bit, in place, reduced and the two D2Q9 forms.
+inline int best_shape(lbmp_handle* h, int tiles, int nmarch, const MarchCost* cost, const double* scale,
+                      const int* per_sm, int n, int sms, int& chunk)
+{
+    const int key[6] = {tiles, nmarch, h->opt_chunk, h->opt_ctas, per_sm[0], n};
+    if (h->shape[0] == 0 || memcmp(key, h->shape_for, sizeof key) != 0) {
+        double best = 0.0;
+        const int c0 = h->opt_chunk > 0 ? (h->opt_chunk < nmarch ? h->opt_chunk : nmarch)
+                                        : (nmarch < kLongestItem ? nmarch : kLongestItem);
+        const int c1 = h->opt_chunk > 0 ? c0 : 1;
+        for (int k = 0; k < n; ++k) {
+            const int per = (h->opt_ctas > 0 && h->opt_ctas < per_sm[k]) ? h->opt_ctas : per_sm[k];
+            for (int c = c0; c >= c1; --c) {
+                const double t = scale[k] * march_time(cost[k], tiles, nmarch, c, per, sms);
+                if ((k == 0 && c == c0) || t < best) {
+                    best = t;
+                    h->shape[0] = c;
+                    h->shape[1] = k;
+                }
+            }
+        }
+        memcpy(h->shape_for, key, sizeof key);
+    }
+    chunk = h->shape[0];
+    return h->shape[1];
+}
+inline LaunchShape launch_shape(lbmp_handle* h, const MarchCost& cost, int tiles, int nmarch, int per_sm, int sms)
+{
+    if (per_sm < 1) per_sm = 1;
+    const double one = 1.0;
+    int chunk;
+    best_shape(h, tiles, nmarch, &cost, &one, &per_sm, 1, sms, chunk);
+    return shape_of(h, tiles, nmarch, chunk, per_sm, sms);
+}
+
+// The FP32 D3Q27 step, and which of its two kernels: with f' loaded one plane
+// ahead at per_sm[1] CTAs per SM, or without at per_sm[0].  Loading ahead takes
+// 0.9 of the time per plane and CTA but starts an item with half a plane more,
+// so it wins where the items are long and its smaller grid does not add a
+// round.  Against the rule before and no loading ahead: 2.1 % less time on
+// average (the best measured choices: 3.6 %) and at most 2 % more for all but
+// 7 of 238 domains; 72^3 48.3 -> 42.8 us, 112^3 141 -> 132, 128^3 192 -> 183.
+constexpr MarchCost kCostFp32[2] = {{1.25, 0.4, 0.0}, {1.25, 0.9, 0.0}};
+constexpr double kScaleFp32[2] = {1.0, 0.9};
+inline LaunchShape launch_shape_ahead(lbmp_handle* h, int tiles, int nmarch, const int per_sm[2], int sms,
+                                      bool& ahead)
+{
+    int chunk;
+    ahead = best_shape(h, tiles, nmarch, kCostFp32, kScaleFp32, per_sm, 2, sms, chunk) != 0;
+    return shape_of(h, tiles, nmarch, chunk, per_sm[ahead], sms);
+}
+
+// Planes (rows) per work item of `n` domains stepped by one batch launch, domain
+// k with tiles[k] tiles marching through nmarch[k] planes, on `slots` resident
+// CTAs (and of the observables' march).  Where 8 or more planes per item leave
+// 2.5 rounds of the full grid, the largest power-of-two part of the longest
+// domain that does: each item stages two planes more than it updates, so longer
+// items win until the rounds get coarse.  Smaller work cannot fill 2.5 rounds;
+// there the time is about rounds x (planes + 1.5) x (0.7 + occupancy), the stages
+// of one item times a stage's latency, which grows with the number of CTAs that
+// share an SM, and the rule takes the planes that make it smallest.
 inline int planes_per_item(const int* tiles, const int* nmarch, int n, long long slots)
 {
     int longest = 1;
@@ -110,89 +208,6 @@ inline int planes_per_item(const int* tiles, const int* nmarch, int n, long long
         }
     }
     return chunk;
-}
-
-// Launch shape of a persistent fused kernel over `tiles` tiles marching
-// through `nmarch` planes (rows in 2-D): planes per work item and grid size,
-// from the handle's options or the defaults.
-struct LaunchShape {
-    int chunk, nitems, grid;
-    bool half_empty;  // the grid takes at most half of the GPU's slots
-};
-inline LaunchShape launch_shape(const lbmp_handle* h, int tiles, int nmarch, int per_sm, int sms)
-{
-    if (per_sm < 1) per_sm = 1;
-    const int ctas = (h->opt_ctas > 0 && h->opt_ctas < per_sm) ? h->opt_ctas : per_sm;
-    const long long cap = (long long)ctas * sms;
-    LaunchShape L;
-    if (h->opt_chunk > 0)
-        L.chunk = h->opt_chunk < nmarch ? h->opt_chunk : nmarch;
-    else
-        L.chunk = planes_per_item(&tiles, &nmarch, 1, (long long)per_sm * sms);
-    L.nitems = tiles * ((nmarch + L.chunk - 1) / L.chunk);
-    L.grid = (int)(L.nitems < cap ? L.nitems : cap);
-    L.half_empty = 2LL * L.grid <= (long long)per_sm * sms;
-    return L;
-}
-
-// Estimated time of a launch of `tiles` tiles marching through `nmarch` planes
-// in items of `chunk` planes, on per_sm CTAs of each of `sms` SMs, in units of
-// its own kernel: a plane takes 1.25 + the CTAs that share the SM, an item
-// `extra` planes more than it updates.  In the first rounds the slots run in
-// step, so the time is that of the rounds, the last one with the CTAs that are
-// left; later the slots have drifted apart and the time tends to the mean load.
-inline double march_time(int tiles, int nmarch, int chunk, int per_sm, int sms, double extra)
-{
-    const int per_tile = (nmarch + chunk - 1) / chunk;
-    const long long slots = (long long)per_sm * sms, items = (long long)tiles * per_tile;
-    const long long rounds = (items + slots - 1) / slots;
-    const double full = 1.25 + per_sm, last = 1.25 + (double)(items - (rounds - 1) * slots) / sms;
-    const double in_step = (chunk + extra) * ((double)(rounds - 1) * full + last);
-    const double mean = (double)tiles * (nmarch + extra * per_tile) / (double)slots * full;
-    const double least = (chunk + extra) * (rounds == 1 ? last : full);
-    const double w = std::exp(-0.4 * (double)(rounds - 1));
-    return w * in_step + (1.0 - w) * (mean > least ? mean : least);
-}
-
-// Launch shape of the FP32 D3Q27 step, and which of its two kernels: with f'
-// loaded one plane ahead at per_sm[1] CTAs per SM, or without at per_sm[0].
-// Loading ahead takes 0.9 of the time per plane and CTA but starts an item with
-// half a plane more, so it wins where the items are long and its smaller grid
-// does not add a round.  The estimates' constants are the best of a grid over
-// 238 domains from 24^3 to 384x384x192 with every chunk measured: against 32
-// planes halved until 2.5 rounds are full, without loading ahead, 2.1 % less time on
-// average (the best measured choices: 3.6 %) and at most 2 % more for all but
-// 7 of them; 72^3 48.3 -> 42.8 us, 112^3 141 -> 132, 128^3 192 -> 183.
-inline LaunchShape launch_shape_ahead(lbmp_handle* h, int tiles, int nmarch, const int per_sm[2], int sms,
-                                      bool& ahead)
-{
-    const int key[3] = {nmarch, h->opt_chunk, h->opt_ctas};
-    if (h->shape[0] == 0 || memcmp(key, h->shape_for, sizeof key) != 0) {  // 128 estimates: once per handle and options
-        double best = 0.0;
-        const int c0 = h->opt_chunk > 0 ? (h->opt_chunk < nmarch ? h->opt_chunk : nmarch) : nmarch < 64 ? nmarch : 64;
-        const int c1 = h->opt_chunk > 0 ? c0 : 1;
-        for (int k = 0; k < 2; ++k) {
-            const int per = (h->opt_ctas > 0 && h->opt_ctas < per_sm[k]) ? h->opt_ctas : per_sm[k];
-            for (int c = c0; c >= c1; --c) {
-                const double t = (k ? 0.9 : 1.0) * march_time(tiles, nmarch, c, per, sms, k ? 0.9 : 0.4);
-                if ((k == 0 && c == c0) || t < best) {
-                    best = t;
-                    h->shape[0] = c;
-                    h->shape[1] = per;
-                    h->shape[2] = k;
-                }
-            }
-        }
-        memcpy(h->shape_for, key, sizeof key);
-    }
-    LaunchShape L;
-    L.chunk = h->shape[0];
-    ahead = h->shape[2] != 0;
-    const long long cap = (long long)h->shape[1] * sms;
-    L.nitems = tiles * ((nmarch + L.chunk - 1) / L.chunk);
-    L.grid = (int)(L.nitems < cap ? L.nitems : cap);
-    L.half_empty = 2LL * L.grid <= (long long)per_sm[ahead] * sms;
-    return L;
 }
 
 // Launch of a step kernel that begins with after_previous().  A grid that
