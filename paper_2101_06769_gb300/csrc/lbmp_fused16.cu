@@ -18,13 +18,15 @@
 //   * the ghost plane beyond a wall (mirrored phi, reading A17) is a copy of
 //     the wall plane's phi instead of a second staging of that plane.
 // What bounds it: instruction issue (every value is decoded and encoded; DRAM
-// stands at a fifth of its rate) and the instruction cache.  It issues
-// 3002 instructions per cell (3553 when g codes were staged as 32-bit words, the
-// two population sets were emitted in two passes and divisions were the
-// compiler's): 1.09 ms per step on the 128x128x512 RT workload in FP16 (1.21
-// before), BF16 1.07 (1.18).  With the
-// ring's codes loaded beside the others (400 B of spills) 1.22, at four CTAs
-// per SM (500 B of spills) 1.12.
+// stands at a quarter of its rate) and the instruction cache.  It issues 3002
+// instructions per cell (3553 when g codes were staged as 32-bit words, the two
+// population sets were emitted in two passes and divisions were the
+// compiler's).  128x128x512 RT workload, FP16 / BF16: 1.00 / 0.99 ms per step;
+// 1.05 / 1.03 with a second barrier per plane (three phi planes in rotation);
+// 1.21 / 1.18 before all of these.  The ring's codes loaded beside the others
+// spill (480 B) wherever their decoding is put: 1.09-1.14; one decoding loop run
+// over the own and the ring cell, 500 instructions of code less, 1.02; four
+// CTAs per SM (500 B of spills) 1.12.
 #define LBMP_TILE_NS tile16
 #ifndef LBMP_FUSED_BYTEOFF
 #define LBMP_FUSED_BYTEOFF 2
@@ -67,7 +69,7 @@ struct EncCell {
 
 constexpr int C3 = 13;
 constexpr int GX = TX + 4, GY = TY + 4, GPLANE = GX * GY;  // g reference plane: tile + two rings
-constexpr size_t kSmem16 = sizeof(float2) * 3 * PLANE + sizeof(float) * (2 * Q3 * NT + 4 * GPLANE + 4 * PLANE) +
+constexpr size_t kSmem16 = sizeof(float2) * 4 * PLANE + sizeof(float) * (2 * Q3 * NT + 4 * GPLANE + 4 * PLANE) +
                            sizeof(int) * (GPLANE + PLANE);
 
 struct DirPtrs16 {
@@ -266,8 +268,8 @@ template <class St>
 __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtrs16& Dp, const ThreadGeo& T,
                                                 float* smem, int x0, int y0, int z0, int z1)
 {
-    float2* phiS = (float2*)smem;                // (hi, lo) [3][PLANE]
-    float* gS = (float*)(phiS + 3 * PLANE);      // [2][27][NT] decoded own g
+    float2* phiS = (float2*)smem;                // (hi, lo) [4][PLANE]
+    float* gS = (float*)(phiS + 4 * PLANE);      // [2][27][NT] decoded own g
     float* RG = gS + 2 * Q3 * NT;                // [4][GPLANE] g references
     float* RF = RG + 4 * GPLANE;                 // [4][PLANE] f' references
     int* offG = (int*)(RF + 4 * PLANE);
@@ -288,18 +290,21 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
     load_ref_plane(p, Dp.rgin, z0 - 1, RG, GPLANE, offG, tid);
     load_ref_plane(p, Dp.rgin, z0, RG, GPLANE, offG, tid);
     load_ref_plane(p, Dp.rfin, z0 - 1, RF, PLANE, offF, tid);
-    int sP = 0, sC = 1, sN = 2;
+    // One barrier per plane: phi and the references have four planes in rotation,
+    // so what a thread that has passed the barrier of plane z writes for plane
+    // z+2 is what no thread reads any more after that barrier.
+    const auto phi_at = [&](int zz) { return phiS + ((zz - z0 + 1) & 3) * PLANE; };
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) {  // planes z0 - 1 and z0
         S.load_g(z0 - 1 + k, qo);
         cp_async_commit();
         cp_async_wait_all();
         __syncthreads();
-        S.finish(z0 - 1 + k, qo, gS + (k ^ 1) * Q3 * NT, phiS + (k ? sC : sP) * PLANE);
+        S.finish(z0 - 1 + k, qo, gS + (k ^ 1) * Q3 * NT, phi_at(z0 - 1 + k));
         S.issue_refs(z0 - 1 + k);
     }
     cp_async_wait_all();
-    if (ghost_plane(p, z0 - 1)) S.copy_phi(phiS + sC * PLANE, phiS + sP * PLANE);
+    if (ghost_plane(p, z0 - 1)) S.copy_phi(phi_at(z0), phi_at(z0 - 1));
     __syncthreads();
     for (int z = z0; z < z1; ++z) {
         const int cur = (z - z0) & 1;
@@ -312,8 +317,8 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
         {
             unsigned short q[Q3];
             load_codes(Dp.fin, own, P, q);
-            S.finish(z + 1, qo, gS + (cur ^ 1) * Q3 * NT, phiS + sN * PLANE);
-            if (ghost_plane(p, z + 1)) S.copy_phi(phiS + sC * PLANE, phiS + sN * PLANE);
+            S.finish(z + 1, qo, gS + (cur ^ 1) * Q3 * NT, phi_at(z + 1));
+            if (ghost_plane(p, z + 1)) S.copy_phi(phi_at(z), phi_at(z + 1));
             float fr[Q3];
             if (P.lo || P.hi)
                 S.template decode_f<true>(z, P.lo, P.hi, q, fr);
@@ -324,9 +329,9 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
         cp_async_wait_all();
         __syncthreads();
         if (valid) {
-            const float2* pm = phiS + sP * PLANE + T.oslot;
-            const float2* pc = phiS + sC * PLANE + T.oslot;
-            const float2* pn = phiS + sN * PLANE + T.oslot;
+            const float2* pm = phi_at(z - 1) + T.oslot;
+            const float2* pc = phi_at(z) + T.oslot;
+            const float2* pn = phi_at(z + 1) + T.oslot;
             const float2 centre = pc[0];
             float grad[3], lap, inv_rho, nu, dh[27];
             repro::stencil_from<3>(
@@ -347,12 +352,8 @@ __device__ __forceinline__ void fused_segment16(const DevParams& p, const DirPtr
                 EncCell<St>{Dp.fout, Dp.rfout, self, off_f, 0.f, code_seed(p, elem_index(self), 0)},
                 EncCell<St>{Dp.gout, Dp.rgout, self, off_g, 0.f, code_seed(p, elem_index(self), 1)});
         }
-        __syncthreads();
-        const int t = sP;
-        sP = sC;
-        sC = sN;
-        sN = t;
     }
+    __syncthreads();  // the caller may reuse shared memory
 }
 
 template <class St>
