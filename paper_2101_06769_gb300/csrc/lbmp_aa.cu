@@ -15,11 +15,18 @@
 // phi = sum g is formed by the phase-aware phi pass of lbmp_kernels.cu
 // before the step (the two-set kernels form it from the g they stage, ring
 // cells included; here a ring cell's slots may already hold its owner's
-// post-collision values).  The step stages phi of three planes (tile and
-// ring) from that array and the tile's own g one plane ahead; the per-cell
-// arithmetic is that of the two-set kernels (here the phase-field outputs first,
-// then the relaxation and the flow), so the results equal
-// them to within the rounding of separately compiled units.
+// post-collision values).  The step stages phi (tile and ring) from that array
+// and the tile's own g one plane ahead, keeps the layer sums of three planes in
+// registers and loads f' one plane ahead (a cell's slots are written by that
+// cell alone); the per-cell arithmetic is that of the two-set kernels, so the
+// results equal them to within the rounding of separately compiled units.
+// What bounds it: memory latency and the accesses' pattern (an odd step's loads
+// and stores are both shifted; the phi pass reads g once more): 128x128x512 RT
+// workload 0.973 ms per step, 200x180x160 0.727 ms, 64^3 33 us; 1.010, 0.759
+// and 35 with three phi planes, two barriers per plane, the outputs in two
+// passes and f' loaded in its own plane.  Without loading ahead 1.002, at four
+// CTAs per SM without it 0.980 (64^3 35 us).  Element indices: a state of 2^30
+// cells fits the memory, its arrays no 32-bit byte offset.
 #define LBMP_TILE_NS tile_aa
 #define LBMP_FUSED_MINB 3
 #define LBMP_OUT_ORDERED 1
@@ -135,80 +142,96 @@ __device__ __forceinline__ void stage_g(const DevParams& p, const AAPtrs& D, con
 
 template <bool Odd, bool Walls>
 __device__ __forceinline__ void collide_cell(const DevParams& p, const AAPtrs& D, const Column& own, const Plane& P,
-                                             const float2* pm, const float2* pc, const float2* pn, const FlowMoments& m,
-                                             float* gcol)
+                                             const LayerSums& below, const LayerSums& here, const LayerSums& above,
+                                             const FlowMoments& m, const float* gcol)
 {
-    const float2 centre = pc[0];
     float grad[3], lap;
-    stencil_from<3>(
-        [&](int a) {
-            const int cz = Lat<3>::cz(a);
-            return (cz < 0 ? pm : (cz == 0 ? pc : pn))[Lat<3>::cy(a) * RX + Lat<3>::cx(a)];
-        },
-        grad, lap);
+    stencil_from_layers<3>(below, here, above, grad, lap);
     CellState s;
     float inv_rho, nu;
-    flow_closure<3>(p, centre.x, grad, lap, m, s, inv_rho, nu);
-    phase_outputs<3>(p, s, GFromStrided{gcol, NT}, centre.x, centre.y, AAOut<Odd, Walls>{D.g, own, P});
     Residual R;
+    flow_closure<3>(p, here.c.x, grad, lap, m, s, inv_rho, nu);
+    const AAOut<Odd, Walls> fo{D.f, own, P}, go{D.g, own, P};
     flow_relax<3>(m, s, inv_rho, nu, R);
-    flow_outputs<3>(p, s, R, m, AAOut<Odd, Walls>{D.f, own, P});
+    collide_outputs<3>(p, s, R, m, GFromStrided{gcol, NT}, here.c.x, here.c.y, fo, go);
 }
 
-// planes [z0, z1) of the tile at (x0, y0); ends with a barrier
+// planes [z0, z1) of the tile at (x0, y0); ends with a barrier.  One barrier per
+// plane: the phi of plane z+1 goes to the slot whose plane was last read before
+// the previous plane's barrier (its layer sums stay in registers), and g is
+// private to its thread.
 template <bool Odd>
 __device__ __forceinline__ void aa_segment(const DevParams& p, const AAPtrs& D, const float* phi, const ThreadGeo& T,
                                            float* smem, int x0, int y0, int z0, int z1)
 {
-    float2* phiS = (float2*)smem;              // (hi, lo) [3][RY][RX]
-    float* gS = (float*)(phiS + 3 * PLANE);    // [2][27][NT] own g, one plane ahead
+    float2* phiS = (float2*)smem;              // (hi, lo) [2][RY][RX]
+    float* gS = (float*)(phiS + 2 * PLANE);    // [2][27][NT] own g, one plane ahead
     const int tid = T.tid;
     Column own, ring;
     set_column(own, p, pmod(x0 + T.tx, p.nx), pmod(y0 + T.ty, p.ny));
     set_column(ring, p, pmod(x0 + T.lx, p.nx), pmod(y0 + T.ly, p.ny));
     const bool valid = (x0 + T.tx < p.nx) && (y0 + T.ty < p.ny);
-    int sP = 0, sC = 1, sN = 2;
-    stage_phi(p, phi, own, ring, T, z0 - 1, phiS + sP * PLANE);
-    stage_phi(p, phi, own, ring, T, z0, phiS + sC * PLANE);
+    const auto layer = [&](int slot, LayerSums& L) {
+        const float2* c = phiS + slot * PLANE + T.oslot;
+        layer_sums<3>([&](int dx, int dy) { return c[dy * RX + dx]; }, L);
+    };
+    float fr[Q3];
+    const auto load_f = [&](const Plane& P) {
+        if (P.lo || P.hi)
+            Unroll<Q3>::run(AALoad<Odd, true>{D.f, own, P, fr});
+        else
+            Unroll<Q3>::run(AALoad<Odd, false>{D.f, own, P, fr});
+    };
+    stage_phi(p, phi, own, ring, T, z0 - 1, phiS);
+    stage_phi(p, phi, own, ring, T, z0, phiS + PLANE);
+    cp_async_commit();
     stage_g<Odd>(p, D, own, z0, gS + tid);
     cp_async_commit();
+    {
+        Plane P;
+        set_plane(P, p, z0);
+        load_f(P);
+    }
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();
+    LayerSums below, here;
+    layer(0, below);
+    layer(1, here);
+    __syncthreads();
     for (int z = z0; z < z1; ++z) {
         const int cur = (z - z0) & 1;
-        stage_phi(p, phi, own, ring, T, z + 1, phiS + sN * PLANE);
+        stage_phi(p, phi, own, ring, T, z + 1, phiS + cur * PLANE);
         cp_async_commit();  // group: phi of plane z+1 (needed now)
         if (z + 1 < z1) stage_g<Odd>(p, D, own, z + 1, gS + (cur ^ 1) * Q3 * NT + tid);
         cp_async_commit();  // group: g of plane z+1 (needed next iteration)
         Plane P;
         set_plane(P, p, z);
-        float fr[Q3];
-        if (P.lo || P.hi)
-            Unroll<Q3>::run(AALoad<Odd, true>{D.f, own, P, fr});
-        else
-            Unroll<Q3>::run(AALoad<Odd, false>{D.f, own, P, fr});
         FlowMoments m;
         flow_moments<3>(m, fr);
+        {
+            Plane N;
+            set_plane(N, p, z + 1 < z1 ? z + 1 : z);
+            load_f(N);
+        }
         asm volatile("cp.async.wait_group 1;\n" ::: "memory");  // all but the g of plane z+1
         __syncthreads();
+        LayerSums above;
+        layer(cur, above);
         if (valid) {
-            const float2* pm = phiS + sP * PLANE + T.oslot;
-            const float2* pc = phiS + sC * PLANE + T.oslot;
-            const float2* pn = phiS + sN * PLANE + T.oslot;
-            float* gcol = gS + cur * Q3 * NT + tid;
+            const float* gcol = gS + cur * Q3 * NT + tid;
             if (P.lo || P.hi)
-                collide_cell<Odd, true>(p, D, own, P, pm, pc, pn, m, gcol);
+                collide_cell<Odd, true>(p, D, own, P, below, here, above, m, gcol);
             else
-                collide_cell<Odd, false>(p, D, own, P, pm, pc, pn, m, gcol);
+                collide_cell<Odd, false>(p, D, own, P, below, here, above, m, gcol);
         }
-        __syncthreads();  // phi slot and g buffer reuse
-        const int t = sP;
-        sP = sC;
-        sC = sN;
-        sN = t;
+        below = here;
+        here = above;
     }
     cp_async_wait_all();  // nothing of this segment is left in flight
+    __syncthreads();
 }
 
-constexpr size_t kSmemAA = sizeof(float2) * 3 * PLANE + sizeof(float) * 2 * Q3 * NT;
+constexpr size_t kSmemAA = sizeof(float2) * 2 * PLANE + sizeof(float) * 2 * Q3 * NT;
 
 template <bool Odd>
 __global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_aa_kernel(DevParams p, AAArgs A, AAPtrs D)

@@ -2,12 +2,10 @@
 // 16 x 8 tile (a launch shape of the autotuners; kernel source
 // lbmp_fused3_body.cuh).
 // Four CTAs (16 warps) per SM at 128 registers, ring phi from register loads,
-// column and plane offsets in bytes.  On the 128x128x512 RT workload a step
-// takes 0.738 ms (0.820 ms with the earlier arithmetic, which issued 2334
-// instructions per cell, and two barriers per plane).  It no longer follows the
-// instruction count: 3 or 5 CTAs per SM take 0.747 / 0.745 ms, element indices
-// 0.732, a ring staged by cp.async 0.748, a 32 x 8 tile 0.778, and the same
-// access pattern without arithmetic 0.706 ms.
+// column and plane offsets in bytes, f' loaded in its own plane.  On the
+// 128x128x512 RT workload a step takes 0.749 ms (0.736 at 32 x 4):
+// half-warp rows take more L1 and L2 transactions per byte; the smaller
+// ring pays on narrow domains only.
 #define LBMP_FUSED_MINB 4
 #define LBMP_FUSED_BYTEOFF 4
 #define LBMP_FUSED_RINGREG 1
