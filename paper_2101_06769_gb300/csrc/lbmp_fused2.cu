@@ -11,6 +11,13 @@
 // field on the reduced lattice D2Q5 (first-order equilibrium and correction
 // term, Sec. 2.2): 5 staged g values, and the stored previous phi u of the
 // staged row copied with them.
+// What bounds it: at large sizes DRAM (4096x2048 0.227 ms per step, 79 % of the
+// copy rate; 0.264 with the earlier arithmetic and 7 CTAs per SM), at small ones
+// the latency of a row's loads and the launch (64x256 3.4 us).  Loading f'
+// one row ahead or g two rows ahead 0.239-0.243, the stencil by layers 0.229 at
+// the cost of 5 % at small sizes (a second barrier's worth of set-up).  The
+// symmetry axis keeps the earlier arithmetic (lbmp_repro.cuh): rounding grows
+// quickly in the impacts it serves.
 #include "lbmp_internal.h"
 #include "lbmp_repro.cuh"
 
