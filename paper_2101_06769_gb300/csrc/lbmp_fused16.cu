@@ -17,16 +17,17 @@
 //     one plane later.
 //   * the ghost plane beyond a wall (mirrored phi, reading A17) is a copy of
 //     the wall plane's phi instead of a second staging of that plane.
-// What bounds it: instruction issue (every value is decoded and encoded; DRAM
-// stands at a quarter of its rate) and the instruction cache.  It issues 3002
-// instructions per cell (3553 when g codes were staged as 32-bit words, the two
-// population sets were emitted in two passes and divisions were the
-// compiler's).  128x128x512 RT workload, FP16 / BF16: 1.00 / 0.99 ms per step;
-// 1.05 / 1.03 with a second barrier per plane (three phi planes in rotation);
-// 1.21 / 1.18 before all of these.  The ring's codes loaded beside the others
-// spill (480 B) wherever their decoding is put: 1.09-1.14; one decoding loop run
-// over the own and the ring cell, 500 instructions of code less, 1.02; four
-// CTAs per SM (500 B of spills) 1.12.
+// What bounds it: instruction issue (58 % of the slots; every value is decoded
+// and encoded; DRAM stands at a quarter of its rate) and the instruction cache,
+// the first of its stalls.  128^3 FP16 issues 2741 instructions per cell (3553
+// when g codes were staged as 32-bit words, the two population sets were emitted
+// in two passes, divisions were the compiler's and items had 8 planes).
+// 128x128x512 RT workload, FP16 / BF16: 1.00 / 0.99 ms per step; 1.05 / 1.03
+// with a second barrier per plane (three phi planes in rotation); 1.21 / 1.18
+// before all of these.  The ring's codes loaded beside the others spill (480 B)
+// wherever their decoding is put: 1.09-1.14; one decoding loop run over the own
+// and the ring cell, 500 instructions of code less, 1.02; four CTAs per SM (500 B
+// of spills) 1.12.
 #define LBMP_TILE_NS tile16
 #ifndef LBMP_FUSED_BYTEOFF
 #define LBMP_FUSED_BYTEOFF 2

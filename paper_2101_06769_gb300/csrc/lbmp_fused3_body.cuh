@@ -180,7 +180,10 @@ __device__ __forceinline__ void stage_finish(int tid, int oslot, int rslot, cons
 // 2.58 -> 2.52 ms, 160^3 0.377 -> 0.363 ms; where a step is a few planes per
 // CTA the fourth CTA is worth more (48^3 14.7 -> 16.5 us, 32^3 6.9 -> 7.4 us),
 // and so it is to batches (3.7 M cells 324 -> 330 us) and the reduced phase
-// lattice (0.447 -> 0.458 ms).  At two CTAs per SM 0.760 ms.
+// lattice (0.447 -> 0.458 ms).  At two CTAs per SM 0.760 ms.  128^3: 1610
+// instructions per cell, 49 % of the issue slots, long scoreboard first of the
+// stalls; a smaller or larger shared memory carveout changes nothing (0.717, 0.722
+// at 164 KiB).
 template <bool Ahead>
 __device__ __forceinline__ void fused_segment(const DevParams& p, const DirPtrs& Dp, const ThreadGeo& T, float* smem,
                                               int x0, int y0, int z0, int z1, float* __restrict__ phiu)
