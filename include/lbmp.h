@@ -185,9 +185,10 @@ typedef struct lbmp_handle lbmp_handle;
  * and g, the stored previous phi u of the reduced phase lattice, the stored
  * velocities of LBMP_FLAG_DIVU, a phi field (8 bytes per cell) only for the
  * reference pair (LBMP_OPT_KERNEL = 1, or LBMP_FLAG_DIVU), and a few KiB for
- * the observables; no device work.  The fused kernels never store phi: the
- * observables and lbmp_get_state form it in the population set the next
- * step overwrites.  Errors: INVALID_ARG (bad grid or parameters), NOMEM,
+ * the observables; no device work.  The fused kernels never store phi, nor do
+ * the observables of FP32 D3Q27 domains; those of other forms and
+ * lbmp_get_state form it in the population set the next step overwrites.
+ * Errors: INVALID_ARG (bad grid or parameters), NOMEM,
  * CUDA.  The caller owns *out and releases it with lbmp_destroy. */
 LBMP_API int lbmp_create(const lbmp_grid *grid, lbmp_lattice lattice, const lbmp_params *params,
                 void *cuda_stream, lbmp_handle **out);
