@@ -322,9 +322,11 @@ __global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_batchg3_kernel(const
 // by layers, f' and the closure; the running sums stay in registers.  Reads
 // each population once and stores no phi array, where a phi pass and a pass of
 // 27-neighbour gathers over its (hi, lo) arrays read 2.3 times the bytes and
-// spent most of their time on index divisions and FP64 instructions: 1.92 ->
-// 0.444 ms on 128x128x512, 1.81 GB read at 4.1 TB/s (5 CTAs per SM, with
-// spills: 0.475).  Grid-strided work items, partial sums per CTA in
+// spent most of their time on index divisions and gathers: 1.92 -> 0.49 ms on
+// 128x128x512, 1.81 GB read at 3.7 TB/s.  The sums are FP64 per cell (ObsAcc);
+// in pairs of FP32 values the call takes 0.45 ms instead of 0.50, but a
+// thread's sum loses 1e-12 over thousands of cells, and |u| above 1e19 or
+// below 1e-16 leaves the range.  Grid-strided work items, partial sums per CTA in
 // a fixed order (deterministic).  cols: phi on the spike column (nx/2, ny/2)
 // and the bubble column (0, 0), or null.
 __device__ __forceinline__ void obs_phi(const DevParams& p, const DirPtrs& D, const Column& own, const Column& ring,
