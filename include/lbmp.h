@@ -339,7 +339,9 @@ typedef struct lbmp_batch lbmp_batch;
 
 /* hbm_budget: upper bound (bytes) on the summed device state of the members,
  * 0 = none; cuda_stream: stream of all batch work (NULL: the batch creates a
- * private stream, since the legacy default stream cannot be captured). */
+ * private stream, since the legacy default stream cannot be captured).  In a
+ * batch of D3Q27 and D2Q9 members the D2Q9 kernels run on a second stream, one
+ * priority level above cuda_stream (at the same level if that is the greatest). */
 LBMP_API int lbmp_batch_create(size_t hbm_budget, void *cuda_stream, lbmp_batch **out);
 LBMP_API int lbmp_batch_destroy(lbmp_batch *b);
 /* Admit h for `steps` more steps (> 0).  Members may be D2Q9 or D3Q27

@@ -299,12 +299,11 @@ LBMP_API int lbmp_batch_create(size_t hbm_budget, void* cuda_stream, lbmp_batch*
         b->own_stream = e == cudaSuccess;
     }
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
-    // the D2Q9 members' branch goes first where both have CTAs to place: the
-    // D3Q27 kernels fill every slot of the GPU, and the few short 2-D items
-    // would otherwise start when those end
-    int least = 0, greatest = 0;
+    int own = 0, least = 0, greatest = 0;
+    if (e == cudaSuccess) e = cudaStreamGetPriority(b->stream, &own);
     if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->side, cudaStreamNonBlocking, greatest);
+    if (e == cudaSuccess)
+        e = cudaStreamCreateWithPriority(&b->side, cudaStreamNonBlocking, lbmp::branch_priority(own, greatest));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_table, sizeof(lbmp::BatchDomain) * kMaxMembers);

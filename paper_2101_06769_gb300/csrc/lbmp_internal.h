@@ -210,6 +210,16 @@ inline int planes_per_item(const int* tiles, const int* nmarch, int n, long long
     return chunk;
 }
 
+// Priority of a batch's second branch (its D2Q9 members): one level above the
+// batch's stream, so that its few short items go before the D3Q27 kernels of the
+// same step, which fill every slot of the GPU (they would otherwise start when
+// those end), and no further before the caller's other work.  (Smaller numbers are
+// greater priorities.)
+inline int branch_priority(int stream_priority, int greatest)
+{
+    return stream_priority > greatest ? stream_priority - 1 : greatest;
+}
+
 // Launch of a step kernel that begins with after_previous().  A grid that
 // leaves at least half of the GPU's slots empty is launched while the kernel
 // before it in the stream still runs (also as an edge of a captured graph): on
