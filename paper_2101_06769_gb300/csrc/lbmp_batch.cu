@@ -52,8 +52,6 @@ enum Kind {
     kKinds = 10
 };
 constexpr int kLast3 = kF32x3R;  // the D3Q27 kinds are kF32x3 .. kLast3
-// resident CTAs per SM of each kind's kernel
-constexpr int kCtas[kKinds] = {4, 3, 3, 4, 8, 6, 6, 8, 7, 7};
 
 int kind_of(const lbmp_handle* h)
 {
@@ -116,6 +114,19 @@ const lbmp::Batch3Ops& ops3_of(const lbmp_batch* b, int kind)
     if (kind == kF16x2) return lbmp::batch2_ops_f16;
     if (kind == kBF16x2) return lbmp::batch2_ops_bf16;
     return lbmp::batch3_ops(b->tile);
+}
+
+// attributes of a kind's kernel, and the CTAs of it that one SM holds (not
+// capturable: call before capture)
+cudaError_t prepare(const lbmp_batch* b, int kind, int& per_sm)
+{
+    switch (kind) {
+    case kF32x2: return lbmp::prepare_batch2(b->device, false, false, per_sm);
+    case kF32x2R: return lbmp::prepare_batch2(b->device, true, false, per_sm);
+    case kF32x2S: return lbmp::prepare_batch2(b->device, false, true, per_sm);
+    case kF32x2RS: return lbmp::prepare_batch2(b->device, true, true, per_sm);
+    default: return ops3_of(b, kind).prepare(b->device, per_sm);
+    }
 }
 
 // the kernels of one kind of D3Q27 members: the member-grid form in groups
@@ -191,6 +202,7 @@ cudaError_t rebuild(lbmp_batch* b, bool graphs = true)
 {
     drop_graphs(b);
     b->h_table.clear();
+    cudaError_t e = cudaSuccess;
     for (int kind = 0; kind < kKinds; ++kind) {
     b->dom0[kind] = (int)b->h_table.size();
     const int D = kind >= kF32x2 ? 2 : 3;
@@ -198,19 +210,22 @@ cudaError_t rebuild(lbmp_batch* b, bool graphs = true)
     const bool fp32_2d = kind == kF32x2 || kind == kF32x2R || kind == kF32x2S || kind == kF32x2RS;
     const int TX = fp32_2d ? lbmp::batch2_tile_x() : ops3_of(b, kind).tile_x;
     const int TY = D == 3 ? ops3_of(b, kind).tile_y : 1;
-    int chunk = b->chunk;
-    if (chunk <= 0) {
-        // a kind's members share one launch: the rule takes them together,
-        // with the CTAs per SM its kernel reaches
-        std::vector<int> tiles, nmarch;
-        for (const Member& m : b->members) {
-            if (m.left <= 0 || kind_of(m.h) != kind) continue;
-            const lbmp_grid& g = m.h->grid;
-            tiles.push_back(((g.nx + TX - 1) / TX) * (D == 3 ? (g.ny + TY - 1) / TY : 1));
-            nmarch.push_back(D == 3 ? g.nz : g.ny);
-        }
-        chunk = lbmp::planes_per_item(tiles.data(), nmarch.data(), (int)tiles.size(), (long long)kCtas[kind] * b->sms);
+    // a kind's members share one launch: the rule takes them together, with
+    // the CTAs per SM that its kernel reaches, up to the 8 its constants were
+    // taken with (the FP32 D2Q9 kernels reach 9: 17.8 us per step of five small
+    // domains with 8 in the rule, 18.8 with 9; 15 of them 38.4 and 39.0, 50 alike)
+    std::vector<int> tiles, nmarch;
+    for (const Member& m : b->members) {
+        if (m.left <= 0 || kind_of(m.h) != kind) continue;
+        const lbmp_grid& g = m.h->grid;
+        tiles.push_back(((g.nx + TX - 1) / TX) * (D == 3 ? (g.ny + TY - 1) / TY : 1));
+        nmarch.push_back(D == 3 ? g.nz : g.ny);
     }
+    int chunk = b->chunk, per_sm = 1;
+    if (!tiles.empty() && e == cudaSuccess) e = prepare(b, kind, per_sm);
+    if (chunk <= 0)
+        chunk = lbmp::planes_per_item(tiles.data(), nmarch.data(), (int)tiles.size(),
+                                      (long long)(per_sm < 8 ? per_sm : 8) * b->sms);
     for (const Member& m : b->members) {
         if (m.left <= 0 || kind_of(m.h) != kind) continue;
         const lbmp_handle* h = m.h;
@@ -239,16 +254,7 @@ cudaError_t rebuild(lbmp_batch* b, bool graphs = true)
     b->nitems[kind] = item;
     }
     const int ndom = total_dom(b);
-    cudaError_t e = cudaSuccess;
     if (ndom > 0) {
-        for (int k = kF32x3; k <= kLast3 && e == cudaSuccess; ++k)
-            if (b->ndom[k]) e = ops3_of(b, k).prepare(b->device);
-        if (e == cudaSuccess && b->ndom[kF32x2]) e = lbmp::prepare_batch2(b->device, false, false);
-        if (e == cudaSuccess && b->ndom[kF32x2R]) e = lbmp::prepare_batch2(b->device, true, false);
-        if (e == cudaSuccess && b->ndom[kF32x2S]) e = lbmp::prepare_batch2(b->device, false, true);
-        if (e == cudaSuccess && b->ndom[kF32x2RS]) e = lbmp::prepare_batch2(b->device, true, true);
-        for (int k = kF16x2; k <= kBF16x2 && e == cudaSuccess; ++k)
-            if (b->ndom[k]) e = ops3_of(b, k).prepare(b->device);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(b->d_table, b->h_table.data(), sizeof(lbmp::BatchDomain) * ndom,
                                 cudaMemcpyHostToDevice, b->stream);

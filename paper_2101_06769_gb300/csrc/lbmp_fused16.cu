@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(NT, LBMP_FUSED_MINB) step_batch3s_kernel(const
 
 template <class St>
 struct BatchCfg16 {
-    static int dev, cap;
-    static cudaError_t prepare(int device)
+    static int dev, cap, ctas;
+    static cudaError_t prepare(int device, int& per_sm_out)
     {
         if (dev != device) {
             cudaError_t e = cudaFuncSetAttribute(step_batch3s_kernel<St>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -451,9 +451,11 @@ struct BatchCfg16 {
             if (e != cudaSuccess) return e;
             e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
             if (e != cudaSuccess) return e;
-            cap = (per_sm > 0 ? per_sm : 1) * sms;
+            ctas = per_sm > 0 ? per_sm : 1;
+            cap = ctas * sms;
             dev = device;
         }
+        per_sm_out = ctas;
         return cudaSuccess;
     }
     static cudaError_t launch(const BatchDomain* table, int ndom, int nitems, int device, cudaStream_t stream)
@@ -469,6 +471,8 @@ template <class St>
 int BatchCfg16<St>::dev = -1;
 template <class St>
 int BatchCfg16<St>::cap = 0;
+template <class St>
+int BatchCfg16<St>::ctas = 0;
 
 struct Cfg16 {
     int device = -1;

@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(TX2) step_batch2_kernel(const BatchDomain* __r
 // launch configuration per phase lattice and x boundary [PR + 2 SX] of the
 // single-domain and of the batch kernel
 int g_f2_dev[4] = {-1, -1, -1, -1}, g_f2_per_sm[4] = {0, 0, 0, 0}, g_f2_sms[4] = {0, 0, 0, 0},
-    g_b2_dev[4] = {-1, -1, -1, -1}, g_b2_cap[4] = {0, 0, 0, 0};
+    g_b2_dev[4] = {-1, -1, -1, -1}, g_b2_per_sm[4] = {0, 0, 0, 0}, g_b2_sms[4] = {0, 0, 0, 0};
 
 constexpr MarchCost kCost = {3.0, 1.25, 6.0};
 
@@ -414,17 +414,13 @@ cudaError_t launch_step_fused2(lbmp_handle* h)
     }
 }
 
-cudaError_t prepare_batch2(int device, bool reduced, bool sym)
+cudaError_t prepare_batch2(int device, bool reduced, bool sym, int& per_sm)
 {
     const int k = (reduced ? 1 : 0) + (sym ? 2 : 0);
     const void* fns[4] = {(const void*)step_batch2_kernel<false, false>, (const void*)step_batch2_kernel<true, false>,
                           (const void*)step_batch2_kernel<false, true>, (const void*)step_batch2_kernel<true, true>};
-    int per_sm = 0, sms = 0, dev = g_b2_dev[k];
-    cudaError_t e = setup_kernel(fns[k], device, dev, per_sm, sms);
-    if (e == cudaSuccess && g_b2_dev[k] != device) {
-        g_b2_cap[k] = per_sm * sms;
-        g_b2_dev[k] = device;
-    }
+    const cudaError_t e = setup_kernel(fns[k], device, g_b2_dev[k], g_b2_per_sm[k], g_b2_sms[k]);
+    per_sm = g_b2_per_sm[k];
     return e;
 }
 
@@ -434,7 +430,8 @@ cudaError_t launch_batch2(const BatchDomain* table, int ndom, int nitems, int de
     const int k = (reduced ? 1 : 0) + (sym ? 2 : 0);
     if (g_b2_dev[k] != device) return cudaErrorNotReady;  // prepare_batch2 first
     if (nitems <= 0) return cudaSuccess;
-    const int grid = nitems < g_b2_cap[k] ? nitems : g_b2_cap[k];
+    const int cap = g_b2_per_sm[k] * g_b2_sms[k];
+    const int grid = nitems < cap ? nitems : cap;
     switch (k) {
     case 0: step_batch2_kernel<false, false><<<grid, TX2, kSmem2, stream>>>(table, ndom, nitems); break;
     case 1: step_batch2_kernel<true, false><<<grid, TX2, kSmem2, stream>>>(table, ndom, nitems); break;

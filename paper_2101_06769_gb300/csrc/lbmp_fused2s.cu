@@ -467,9 +467,11 @@ struct Ops2s {
         D.rgout = h->g[d];
         return launch_after(step_fused2s_kernel<St>, L, TX2, kSmem2s, h->stream, h->dp, A, D);
     }
-    static cudaError_t prepare(int device)
+    static cudaError_t prepare(int device, int& per_sm)
     {
-        return setup2s((const void*)step_batch2s_kernel<St>, device, batch_cfg);
+        const cudaError_t e = setup2s((const void*)step_batch2s_kernel<St>, device, batch_cfg);
+        per_sm = batch_cfg.per_sm;
+        return e;
     }
     static cudaError_t launch(const BatchDomain* table, int ndom, int nitems, int device, cudaStream_t stream)
     {

@@ -463,17 +463,22 @@ cudaError_t launch_batch_epilogue(BatchDomain* table, int ndom, cudaStream_t str
 
 namespace {
 
-int g_batch_dev = -1;
+int g_batch_dev = -1, g_batch_per_sm = 0;
 
-// attributes of the batch kernel (not capturable: call before capture)
-cudaError_t prepare_batch(int device)
+// attributes and occupancy of the batch kernel (not capturable: call before capture)
+cudaError_t prepare_batch(int device, int& per_sm)
 {
     if (g_batch_dev != device) {
-        const cudaError_t e =
+        cudaError_t e =
             cudaFuncSetAttribute(step_batchg3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (e != cudaSuccess) return e;
+        int n = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_batchg3_kernel, NT, kSmemBytes);
+        if (e != cudaSuccess) return e;
+        g_batch_per_sm = n > 0 ? n : 1;
         g_batch_dev = device;
     }
+    per_sm = g_batch_per_sm;
     return cudaSuccess;
 }
 

@@ -307,7 +307,8 @@ bool fused_supported(const lbmp_handle* h);
 // batch kernel of one tile shape of the FP32 D3Q27 fused step
 struct Batch3Ops {
     int tile_x, tile_y;
-    cudaError_t (*prepare)(int device);  // attributes and occupancy (not capturable)
+    // attributes, and the resident CTAs per SM of the kernel (not capturable)
+    cudaError_t (*prepare)(int device, int& per_sm);
     // persistent form (null where a kind has the member-grid form): the
     // members' work items walked by one grid, members read from the device table
     cudaError_t (*launch)(const BatchDomain* table, int ndom, int nitems, int device, cudaStream_t stream);
@@ -342,7 +343,7 @@ cudaError_t launch_step_fused_bulk(lbmp_handle* h);
 // the step kernel(s) selected by LBMP_OPT_KERNEL for this handle (no parity flip)
 cudaError_t launch_step(lbmp_handle* h);
 int batch2_tile_x();
-cudaError_t prepare_batch2(int device, bool reduced, bool sym);  // reduced: D2Q5 phase field; sym: x symmetry axis
+cudaError_t prepare_batch2(int device, bool reduced, bool sym, int& per_sm);  // reduced: D2Q5 phase field; sym: x symmetry axis
 cudaError_t launch_batch2(const BatchDomain* table, int ndom, int nitems, int device, cudaStream_t stream,
                           bool reduced, bool sym);
 cudaError_t launch_batch_epilogue(BatchDomain* table, int ndom, cudaStream_t stream);
