@@ -331,8 +331,9 @@ int lbmp_create_ex(const lbmp_grid* grid, lbmp_lattice lattice, const lbmp_param
     if (N > (1LL << 31) - 1) return fail(LBMP_ERR_INVALID_ARG, "more than 2^31-1 cells");
     if (params->storage != LBMP_FP32 && params->storage != LBMP_FP16_SHIFTED && params->storage != LBMP_BF16_SHIFTED)
         return fail(LBMP_ERR_INVALID_ARG, "unknown storage form");
-    // the D3Q27 16-bit kernel stages codes as 32-bit words holding two
-    // neighbouring cells; the D2Q9 one loads 2-byte codes but keeps the same rule
+    // the interface's rule for 16-bit storage (include/lbmp.h), from kernels that
+    // moved codes as words of two neighbouring cells; the present ones load single
+    // codes, but have run on even widths only
     if (params->storage != LBMP_FP32 && (grid->nx & 1))
         return fail(LBMP_ERR_INVALID_ARG, "16-bit storage needs an even nx");
     if (params->flags & ~63u) return fail(LBMP_ERR_INVALID_ARG, "unknown flag bits");

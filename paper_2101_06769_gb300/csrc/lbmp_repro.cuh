@@ -369,7 +369,7 @@ __device__ __forceinline__ void rest_offsets(const DevParams& p, const CellState
 // (c -> -c, same weight): (a, opp(a)) are the two lanes of the paired FP32
 // arithmetic, and the shared factors (c.u, (c.u)^2, c.G, c.F, c.n) are
 // computed once per pair.
-// dh source: the register array of flow_collide
+// dh source: the register array of flow_relax
 struct DhArray {
     const float* v;
     __device__ __forceinline__ float operator[](int a) const { return v[a]; }
