@@ -176,14 +176,14 @@ __device__ __forceinline__ void stage_finish(int tid, int oslot, int rslot, cons
 // Ahead: f'(z+1) is loaded to registers once the moments of f'(z) are formed, so
 // its latency runs beside the collision and the stores of plane z.  The 27
 // values live across the collision: 168 registers, three CTAs per SM.  Against
-// four CTAs without, on D3Q27 FP32: 128x128x512 0.736 -> 0.715 ms, 384x384x192
-// 2.58 -> 2.52 ms, 160^3 0.377 -> 0.363 ms; where a step is a few planes per
-// CTA the fourth CTA is worth more (48^3 14.7 -> 16.5 us, 32^3 6.9 -> 7.4 us),
-// and so it is to batches (3.7 M cells 324 -> 330 us) and the reduced phase
-// lattice (0.447 -> 0.458 ms).  At two CTAs per SM 0.760 ms.  128^3: 1610
-// instructions per cell, 49 % of the issue slots, long scoreboard first of the
-// stalls; a smaller or larger shared memory carveout changes nothing (0.717, 0.722
-// at 164 KiB).
+// four CTAs without, on D3Q27 FP32 with the default items: 128x128x512 0.738 ->
+// 0.734 ms, 384x384x192 2.643 -> 2.633 ms, 128^3 199 -> 187 us, 72^3 51 -> 46 us.
+// Where a step is a few planes per CTA the fourth CTA is worth more, and so it is
+// to batches and the reduced phase lattice (measured with a cheaper sum in
+// PairOut: 48^3 14.7 -> 16.5 us, 32^3 6.9 -> 7.4 us, batches of 3.7 M cells 324 ->
+// 330 us, reduced 0.447 -> 0.458 ms; two CTAs per SM 0.760 ms on 128x128x512, and
+// another shared memory carveout no change).  128^3: 1640 instructions per cell,
+// 49 % of the issue slots, long scoreboard first of the stalls.
 template <bool Ahead>
 __device__ __forceinline__ void fused_segment(const DevParams& p, const DirPtrs& Dp, const ThreadGeo& T, float* smem,
                                               int x0, int y0, int z0, int z1, float* __restrict__ phiu)

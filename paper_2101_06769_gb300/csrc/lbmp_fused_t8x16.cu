@@ -3,7 +3,7 @@
 // lbmp_fused3_body.cuh).
 // Four CTAs (16 warps) per SM at 128 registers, ring phi from register loads,
 // column and plane offsets in bytes, f' loaded in its own plane.  On the
-// 128x128x512 RT workload a step takes 1.26 ms (0.736 at 32 x 4):
+// 128x128x512 RT workload a step takes 1.30 ms (0.738 at 32 x 4):
 // quarter-warp rows take more L1 and L2 transactions per byte; the smaller
 // ring pays on narrow domains only.
 #define LBMP_FUSED_MINB 4

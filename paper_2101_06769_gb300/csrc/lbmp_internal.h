@@ -165,7 +165,8 @@ inline LaunchShape launch_shape(lbmp_handle* h, const MarchCost& cost, int tiles
 // so it wins where the items are long and its smaller grid does not add a
 // round.  Against the rule before and no loading ahead: 2.1 % less time on
 // average (the best measured choices: 3.6 %) and at most 2 % more for all but
-// 7 of 238 domains; 72^3 48.3 -> 42.8 us, 112^3 141 -> 132, 128^3 192 -> 183.
+// 7 of 238 domains.  With the default items, without loading ahead and now: 72^3
+// 51.2 and 46.1 us, 112^3 144 and 134, 128^3 199 and 187; but 160^3 363 and 401.
 constexpr MarchCost kCostFp32[2] = {{1.25, 0.4, 0.0}, {1.25, 0.9, 0.0}};
 constexpr double kScaleFp32[2] = {1.0, 0.9};
 inline LaunchShape launch_shape_ahead(lbmp_handle* h, int tiles, int nmarch, const int per_sm[2], int sms,
