@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(NT, 4) obs_fused3_kernel(DevParams p, FusedArg
                                                            double* __restrict__ part, double* __restrict__ cols)
 {
     __shared__ float2 phiS[2 * PLANE];
-    __shared__ double sm[4 * (NT / 32)];
+    __shared__ ObsShared<NT> sm;
     const ThreadGeo T = thread_geo();
     const float2* cell = phiS + T.oslot;
     const auto layer = [&](int slot, LayerSums& L) {

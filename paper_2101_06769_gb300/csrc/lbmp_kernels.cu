@@ -651,7 +651,7 @@ template <int D, class St>
 __global__ void __launch_bounds__(256) obs_partial_kernel(DevParams p, Pop<D, St> f, const float* __restrict__ phi,
                                                           double* __restrict__ part, const float* __restrict__ ustore)
 {
-    __shared__ double sm[4 * 8];
+    __shared__ ObsShared<256> sm;
     ObsAcc acc = {};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.N;
          i += (long long)gridDim.x * blockDim.x) {
@@ -820,8 +820,10 @@ struct ObsL {
         const Pop<D, St> f = pop_of<D, St>(h, h->f[h->parity]);
         const float* us = h->uvel[h->parity];  // the velocity the next step's div(u) uses, or null
         const float* phi = phi_buf(h);
-        obs_partial_kernel<D, St><<<h->red_blocks, 256, 0, h->stream>>>(h->dp, f, phi, h->red, us);
-        obs_final_kernel<<<1, 256, 0, h->stream>>>(h->red, h->red_blocks, out);
+        // a block beyond the cells would only reduce zeros
+        const int blocks = (long long)h->red_blocks * 256 < h->N ? h->red_blocks : (int)((h->N + 255) / 256);
+        obs_partial_kernel<D, St><<<blocks, 256, 0, h->stream>>>(h->dp, f, phi, h->red, us);
+        obs_final_kernel<<<1, 256, 0, h->stream>>>(h->red, blocks, out);
         if (full) {
             const int nv = (D == 3) ? h->grid.nz : h->grid.ny;
             const int* pr = h->probe;

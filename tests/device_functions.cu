@@ -7,7 +7,7 @@ using namespace lbmp;
 // every thread of one block takes the same n cells through obs_cell; the block's four sums
 static __global__ void obs_kernel(int n, const float2* phi, const float* rho, const float* u, const float* ph, double* out)
 {
-    __shared__ double sm[4 * 4];
+    __shared__ ObsShared<128> sm;
     ObsAcc acc = {};
     for (int i = 0; i < n; ++i) obs_cell(acc, phi[i], rho[i], u + 3 * i, ph[i]);
     obs_block(acc, sm, out);
